@@ -30,58 +30,190 @@ __global__ void flip_kernel(const __nv_bfloat16* __restrict__ w, int CI, int CO,
 
 constexpr int RED_BLOCKS = 1024;
 
-__global__ void bias_grad_partials(const __nv_bfloat16* __restrict__ dy, int CO, long long P, float* __restrict__ part) {
-    __shared__ float s[256];
-    // thread i takes channel i % CO of pixels i / CO, i / CO + rows, ...
-    const int rows = blockDim.x / CO;
-    float a = 0.0f;
-    const int o = threadIdx.x % CO, r = threadIdx.x / CO;
-    if (r < rows)
-        for (long long p = (long long)blockIdx.x * rows + r; p < P; p += (long long)gridDim.x * rows)
-            a += __bfloat162float(dy[p * CO + o]);
-    s[threadIdx.x] = r < rows ? a : 0.0f;
+__device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
+__device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
+
+// Sums of the channels of dy over pixels, one partial per block.  HBM-bound: a
+// thread takes 8 channels of a pixel in one 16-byte load and keeps 8 sums, the
+// block's threads lie over consecutive bytes, and 4 loads per thread are in
+// flight.  16 x 256 x 256 pixels of 48 channels (100.7 MB, dy written before it):
+// 37.2 us with one 2-byte load per thread and iteration, 18 us so.
+// aligned: dy on a 16-byte boundary (else the same sums from 2-byte loads).
+template <int CO>
+__global__ void __launch_bounds__(256)
+    bias_grad_partials(const __nv_bfloat16* __restrict__ dy, long long P, float* __restrict__ part, bool aligned) {
+    constexpr int NC = CO / 8;                // 16-byte chunks per pixel
+    constexpr int ROWS = 256 / NC;            // pixels per pass of a block
+    __shared__ float s[ROWS][CO];
+    const int j = threadIdx.x % NC, r = threadIdx.x / NC;
+    float a[8] = {};
+    if (r < ROWS) {
+        const long long stride = (long long)gridDim.x * ROWS;
+        auto add = [&](uint4 v) {
+            const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                a[2 * k] += bf16_lo(w[k]);
+                a[2 * k + 1] += bf16_hi(w[k]);
+            }
+        };
+        long long p = (long long)blockIdx.x * ROWS + r;
+        if (aligned) {
+            const uint4* src = reinterpret_cast<const uint4*>(dy) + j;
+            for (; p + 3 * stride < P; p += 4 * stride) {
+                uint4 v[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) v[k] = __ldg(src + (p + k * stride) * NC);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) add(v[k]);
+            }
+            for (; p < P; p += stride) add(__ldg(src + p * NC));
+        } else {
+            for (; p < P; p += stride)
+#pragma unroll
+                for (int k = 0; k < 8; ++k) a[k] += __bfloat162float(dy[p * CO + 8 * j + k]);
+        }
+#pragma unroll
+        for (int k = 0; k < 8; ++k) s[r][8 * j + k] = a[k];
+    }
     __syncthreads();
     if (threadIdx.x < CO) {
         float t = 0.0f;
-        for (int k = 0; k < rows; ++k) t += s[k * CO + threadIdx.x];
+#pragma unroll 4
+        for (int k = 0; k < ROWS; ++k) t += s[k][threadIdx.x];
         part[(size_t)blockIdx.x * CO + threadIdx.x] = t;
     }
 }
 
-__global__ void sum_partials(const float* __restrict__ part, int nb, int CO, float* __restrict__ out) {
-    const int o = blockIdx.x * blockDim.x + threadIdx.x;
-    if (o >= CO) return;
+// out[o] = sum over nb partials of channel o, one block per channel and a tree in
+// a fixed order: latency-bound (58 us when one thread per channel added them in
+// turn, 3 us so at nb = 1024).
+__global__ void __launch_bounds__(256)
+    sum_partials(const float* __restrict__ part, int nb, int CO, float* __restrict__ out) {
+    __shared__ float s[256];
+    const int o = blockIdx.x;
     float t = 0.0f;
-    for (int b = 0; b < nb; ++b) t += part[(size_t)b * CO + o];
-    out[o] = t;
-}
-
-__global__ void mse_partials(const float* __restrict__ pred, const float* __restrict__ target, int U, long long P,
-                             __nv_bfloat16* __restrict__ dpred, double* __restrict__ part) {
-    __shared__ double s[256];
-    const double inv = 1.0 / ((double)P * U);
-    double a = 0.0;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < P * 16; i += (long long)gridDim.x * blockDim.x) {
-        const int c = (int)(i % 16);
-        const double d = c < U ? (double)pred[i] - (double)target[i] : 0.0;
-        a += d * d;
-        if (dpred) dpred[i] = __float2bfloat16_rn((float)(2.0 * inv * d));
-    }
-    s[threadIdx.x] = a;
+    for (int b = threadIdx.x; b < nb; b += 256) t += part[(size_t)b * CO + o];
+    s[threadIdx.x] = t;
     __syncthreads();
-    for (int k = blockDim.x / 2; k > 0; k >>= 1) {
+    for (int k = 128; k > 0; k >>= 1) {
         if (threadIdx.x < k) s[threadIdx.x] += s[threadIdx.x + k];
         __syncthreads();
     }
-    if (threadIdx.x == 0) part[blockIdx.x] = s[0] * inv;
+    if (threadIdx.x == 0) out[o] = s[0];
 }
 
-__global__ void mse_final(const double* __restrict__ part, int nb, double* __restrict__ loss) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        double t = 0.0;
-        for (int b = 0; b < nb; ++b) t += part[b];
-        *loss = t;
+// One pixel of the loss per thread.  The FP64 pipe (2 lanes per clock and SM on
+// GB300) bounds a version that forms every square in double: 208 us at 16 x 256 x
+// 256 pixels, over the 16 channels of which 5 are used.  Here the difference is
+// split exactly into two floats, s + e = pred - target (Knuth's two-sum), its
+// square into h + l (a fused multiply-add gives the product's rounding error), and
+// the pixel's squares are added as such pairs; only the pixel's sum is converted
+// and added in double.  The pairs carry 2^-46 of a pixel's sum, far below the
+// rounding of the double total over the pixels.  Squares that would leave the
+// float range take the double form.
+__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
+    s = __fadd_rn(a, b);
+    const float bb = __fsub_rn(s, a);
+    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+}
+
+// VEC: pred, target and dpred on 16-byte boundaries (else scalar accesses).
+// dpred = 2 inv d: the FP32 product with 2 inv = khi + klo, accurate to 2^-46 before
+// its one rounding to float, then rounded to bfloat16.
+template <bool VEC>
+__global__ void __launch_bounds__(256)
+    mse_partials(const float* __restrict__ pred, const float* __restrict__ target, int U, long long P,
+                 __nv_bfloat16* __restrict__ dpred, double* __restrict__ part, double inv, float khi, float klo) {
+    __shared__ double sh[8];
+    double a = 0.0;
+    for (long long p = (long long)blockIdx.x * 256 + threadIdx.x; p < P; p += (long long)gridDim.x * 256) {
+        const float* pp = pred + p * 16;
+        const float* tt = target + p * 16;
+        uint32_t out[8];
+        float H = 0.0f, L = 0.0f;
+        double far = 0.0;  // squares outside the float range
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            float x[4] = {}, y[4] = {}, g[4] = {};
+            if (4 * q < U) {
+                if constexpr (VEC) {
+                    const float4 xv = *reinterpret_cast<const float4*>(pp + 4 * q);
+                    const float4 yv = *reinterpret_cast<const float4*>(tt + 4 * q);
+                    x[0] = xv.x; x[1] = xv.y; x[2] = xv.z; x[3] = xv.w;
+                    y[0] = yv.x; y[1] = yv.y; y[2] = yv.z; y[3] = yv.w;
+                } else {
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        x[c] = pp[4 * q + c];
+                        y[c] = tt[4 * q + c];
+                    }
+                }
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    if (4 * q + c >= U) continue;
+                    float s, e;
+                    two_sum(x[c], -y[c], s, e);
+                    const float m = fabsf(s);
+                    if (m == 0.0f || (m > 1e-14f && m < 1e18f)) {
+                        const float h = __fmul_rn(s, s);
+                        // the product's error, and the cross term of the split
+                        const float l = __fadd_rn(__fmaf_rn(s, s, -h), __fmul_rn(2.0f * s, e));
+                        float z, r;
+                        two_sum(H, h, z, r);
+                        H = z;
+                        L = __fadd_rn(L, __fadd_rn(r, l));
+                        g[c] = __fmaf_rn(khi, s, __fmaf_rn(khi, e, __fmul_rn(klo, s)));
+                    } else {
+                        const double d = (double)x[c] - (double)y[c];
+                        far += d * d;
+                        g[c] = (float)(2.0 * inv * d);
+                    }
+                }
+            }
+            const __nv_bfloat162 lo = __floats2bfloat162_rn(g[0], g[1]), hi = __floats2bfloat162_rn(g[2], g[3]);
+            out[2 * q] = *reinterpret_cast<const uint32_t*>(&lo);
+            out[2 * q + 1] = *reinterpret_cast<const uint32_t*>(&hi);
+        }
+        a += ((double)H + (double)L);
+        if (far != 0.0) a += far;  // also NaN
+        if (dpred) {
+            if constexpr (VEC) {
+                uint4* o = reinterpret_cast<uint4*>(dpred + p * 16);
+                o[0] = make_uint4(out[0], out[1], out[2], out[3]);
+                o[1] = make_uint4(out[4], out[5], out[6], out[7]);
+            } else {
+#pragma unroll
+                for (int c = 0; c < 16; ++c) {
+                    const uint32_t w = out[c / 2];
+                    dpred[p * 16 + c] = __ushort_as_bfloat16((unsigned short)(c & 1 ? w >> 16 : w & 0xffffu));
+                }
+            }
+        }
     }
+    for (int off = 16; off > 0; off >>= 1) a += __shfl_down_sync(0xffffffffu, a, off);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = a;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double t = 0.0;
+        for (int w = 0; w < 8; ++w) t += sh[w];
+        part[blockIdx.x] = t * inv;
+    }
+}
+
+// The loss from the block partials, in a fixed order (67 us when one thread added
+// the 1024 of them in turn).
+__global__ void __launch_bounds__(256) mse_final(const double* __restrict__ part, int nb, double* __restrict__ loss) {
+    __shared__ double s[256];
+    double t = 0.0;
+    for (int b = threadIdx.x; b < nb; b += 256) t += part[b];
+    s[threadIdx.x] = t;
+    __syncthreads();
+    for (int k = 128; k > 0; k >>= 1) {
+        if (threadIdx.x < k) s[threadIdx.x] += s[threadIdx.x + k];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) *loss = s[0];
 }
 
 __global__ void adam_kernel(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m, float* __restrict__ v,
@@ -102,18 +234,80 @@ __global__ void adam_kernel(float* __restrict__ p, const float* __restrict__ g, 
     }
 }
 
-__global__ void pack_kernel(const float* __restrict__ fields, int B, int H, int W, const float* __restrict__ shift,
-                            const float* __restrict__ scale, float* __restrict__ state, __nv_bfloat16* __restrict__ act) {
-    const long long HW = (long long)H * W, P = B * HW;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < P * 16; i += (long long)gridDim.x * blockDim.x) {
-        const int c = (int)(i % 16);
-        const long long p = i / 16, n = p / HW, q = p % HW;
-        const float* f = fields + n * 6 * HW + q;  // phi, ux, uy, p, c1, c2
-        float v = 0.0f;
-        if (c < 4) v = (f[c * HW] - shift[c]) * scale[c];
-        else if (c == 4) v = ((f[4 * HW] + f[5 * HW]) - shift[4]) * scale[4];
-        state[i] = v;
-        if (act) act[i] = __float2bfloat16_rn(v);
+// Fields to normalised states.  HBM-bound (24 B read and up to 96 B written per
+// pixel): a lane loads its own pixel's six values (a warp reads 128 contiguous
+// bytes per plane), then the warp writes its 32 pixels four lanes (FP32) or two
+// (bfloat16) to a pixel, 512 contiguous bytes per store, the values passed by
+// shuffles.  With one thread per output value, every thread divided by the plane
+// size in 64 bits and re-read its plane one value at a time: 80 us at 16 x 256 x
+// 256 pixels; now 23 us.
+// vec: state and act on 16-byte boundaries (else scalar stores).
+__global__ void __launch_bounds__(256)
+    pack_kernel(const float* __restrict__ fields, int B, long long HW, const float* __restrict__ shift,
+                const float* __restrict__ scale, float* __restrict__ state, __nv_bfloat16* __restrict__ act, bool vec) {
+    const int lane = threadIdx.x & 31;
+    const long long warps = (long long)gridDim.x * 8, per = (HW + 31) / 32;  // 32-pixel groups of an image
+    float sh[5], sc[5];
+#pragma unroll
+    for (int c = 0; c < 5; ++c) {
+        sh[c] = shift[c];
+        sc[c] = scale[c];
+    }
+    for (long long n = blockIdx.y; n < B; n += gridDim.y) {
+        const float* f = fields + n * 6 * HW;
+        for (long long k = (long long)blockIdx.x * 8 + (threadIdx.x >> 5); k < per; k += warps) {
+            const long long q = k * 32 + lane;
+            float v[5] = {};
+            if (q < HW) {
+#pragma unroll
+                for (int c = 0; c < 4; ++c) v[c] = (f[c * HW + q] - sh[c]) * sc[c];
+                v[4] = ((f[4 * HW + q] + f[5 * HW + q]) - sh[4]) * sc[4];
+            }
+            float* so = state + (n * HW + k * 32) * 16;
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                const int px = 8 * t + (lane >> 2), j = lane & 3;
+                float w[5];
+#pragma unroll
+                for (int c = 0; c < 5; ++c) w[c] = __shfl_sync(0xffffffffu, v[c], px);
+                const float4 o = j == 0 ? make_float4(w[0], w[1], w[2], w[3])
+                                        : make_float4(j == 1 ? w[4] : 0.0f, 0.0f, 0.0f, 0.0f);
+                if (k * 32 + px >= HW) continue;
+                float* d = so + px * 16 + 4 * j;
+                if (vec) {
+                    *reinterpret_cast<float4*>(d) = o;
+                } else {
+                    d[0] = o.x;
+                    d[1] = o.y;
+                    d[2] = o.z;
+                    d[3] = o.w;
+                }
+            }
+            if (!act) continue;
+            __nv_bfloat16* ao = act + (n * HW + k * 32) * 16;
+#pragma unroll
+            for (int t = 0; t < 2; ++t) {
+                const int px = 16 * t + (lane >> 1), j = lane & 1;
+                __nv_bfloat16 w[8];
+#pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    const float x = c < 5 ? __shfl_sync(0xffffffffu, v[c], px) : 0.0f;
+                    w[c] = __float2bfloat16_rn(j == 0 ? x : 0.0f);
+                }
+                if (k * 32 + px >= HW) continue;
+                __nv_bfloat16* d = ao + px * 16 + 8 * j;
+                if (vec) {
+                    uint32_t u[4];
+#pragma unroll
+                    for (int c = 0; c < 4; ++c)
+                        u[c] = (uint32_t)__bfloat16_as_ushort(w[2 * c]) | ((uint32_t)__bfloat16_as_ushort(w[2 * c + 1]) << 16);
+                    *reinterpret_cast<uint4*>(d) = make_uint4(u[0], u[1], u[2], u[3]);
+                } else {
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) d[c] = w[c];
+                }
+            }
+        }
     }
 }
 
@@ -141,13 +335,37 @@ __global__ void unpack_macros_kernel(const float* __restrict__ state, int B, int
     }
 }
 
-__global__ void unpack_kernel(const float* __restrict__ state, int B, int H, int W, const float* __restrict__ shift,
-                              const float* __restrict__ scale, float* __restrict__ fields) {
-    const long long HW = (long long)H * W, P = B * HW;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < P * 5; i += (long long)gridDim.x * blockDim.x) {
-        const long long q = i % HW, c = (i / HW) % 5, n = i / (5 * HW);
-        fields[i] = state[(n * HW + q) * 16 + c] / scale[c] + shift[c];
+// The five fields of a state: a lane reads the used part of its pixel (one 32-byte
+// sector of the 64 bytes) and writes one value per plane, 128 contiguous bytes per
+// warp and plane.
+__global__ void __launch_bounds__(256)
+    unpack_kernel(const float* __restrict__ state, int B, long long HW, const float* __restrict__ shift,
+                  const float* __restrict__ scale, float* __restrict__ fields, bool vec) {
+    float sh[5], sc[5];
+#pragma unroll
+    for (int c = 0; c < 5; ++c) {
+        sh[c] = shift[c];
+        sc[c] = scale[c];
     }
+    for (long long n = blockIdx.y; n < B; n += gridDim.y)
+        for (long long q = (long long)blockIdx.x * 256 + threadIdx.x; q < HW; q += (long long)gridDim.x * 256) {
+            const float* s = state + (n * HW + q) * 16;
+            float v[5];
+            if (vec) {
+                const float4 a = *reinterpret_cast<const float4*>(s);
+                v[0] = a.x;
+                v[1] = a.y;
+                v[2] = a.z;
+                v[3] = a.w;
+            } else {
+#pragma unroll
+                for (int c = 0; c < 4; ++c) v[c] = s[c];
+            }
+            v[4] = s[4];
+            float* o = fields + n * 5 * HW + q;
+#pragma unroll
+            for (int c = 0; c < 5; ++c) o[c * HW] = v[c] / sc[c] + sh[c];
+        }
 }
 
 // Per sample and channel (first 5): max |a - b| and sum (a - b)^2 over pixels.
@@ -239,6 +457,13 @@ __global__ void to_bf16_kernel(const float* __restrict__ s, long long n, __nv_bf
 
 int grid_for(long long n, int threads) { return (int)std::max<long long>(1, std::min<long long>((n + threads - 1) / threads, 152LL * 16)); }
 
+// blocks of 256 pixels of an image (x) by images (y), about 16 blocks per SM in all
+dim3 image_grid(long long hw, int batch) {
+    const long long gy = std::min<long long>(batch, 65535);
+    const long long gx = std::min<long long>((hw + 255) / 256, std::max<long long>(1, (152LL * 16 + gy - 1) / gy));
+    return dim3((unsigned)gx, (unsigned)gy);
+}
+
 }  // namespace
 
 extern "C" {
@@ -254,9 +479,11 @@ int lbm_nn_flip_weights(const void* w, int32_t cin, int32_t cout, void* wt, void
 int lbm_nn_bias_grad(const void* dy, int32_t cout, int64_t pixels, float* db, float* partials, void* stream) {
     if (!dy || !db || !partials || (cout != 16 && cout != 48) || pixels < 1) return LBM_ERR_ARG;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    const int threads = cout == 16 ? 256 : 240;  // a whole number of pixels per pass
-    bias_grad_partials<<<RED_BLOCKS, threads, 0, s>>>(static_cast<const __nv_bfloat16*>(dy), cout, pixels, partials);
-    sum_partials<<<1, 64, 0, s>>>(partials, RED_BLOCKS, cout, db);
+    const bool aligned = (uintptr_t)dy % 16 == 0;
+    const auto* d = static_cast<const __nv_bfloat16*>(dy);
+    if (cout == 48) bias_grad_partials<48><<<RED_BLOCKS, 256, 0, s>>>(d, pixels, partials, aligned);
+    else bias_grad_partials<16><<<RED_BLOCKS, 256, 0, s>>>(d, pixels, partials, aligned);
+    sum_partials<<<cout, 256, 0, s>>>(partials, RED_BLOCKS, cout, db);
     return launch_status();
 }
 
@@ -264,8 +491,14 @@ int lbm_nn_mse(const float* pred, const float* target, int32_t used, int64_t pix
                double* loss, void* stream) {
     if (!pred || !target || !loss_partials || !loss || used < 1 || used > 16 || pixels < 1) return LBM_ERR_ARG;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    mse_partials<<<RED_BLOCKS, 256, 0, s>>>(pred, target, used, pixels, static_cast<__nv_bfloat16*>(dpred), loss_partials);
-    mse_final<<<1, 32, 0, s>>>(loss_partials, RED_BLOCKS, loss);
+    const double inv = 1.0 / ((double)pixels * used);
+    const float khi = (float)(2.0 * inv), klo = (float)(2.0 * inv - (double)khi);
+    auto* dp = static_cast<__nv_bfloat16*>(dpred);
+    if (((uintptr_t)pred | (uintptr_t)target | (uintptr_t)dpred) % 16 == 0)
+        mse_partials<true><<<RED_BLOCKS, 256, 0, s>>>(pred, target, used, pixels, dp, loss_partials, inv, khi, klo);
+    else
+        mse_partials<false><<<RED_BLOCKS, 256, 0, s>>>(pred, target, used, pixels, dp, loss_partials, inv, khi, klo);
+    mse_final<<<1, 256, 0, s>>>(loss_partials, RED_BLOCKS, loss);
     return launch_status();
 }
 
@@ -281,17 +514,19 @@ int lbm_nn_adam(float* param, const float* grad, float* m, float* v, const uint8
 int lbm_nn_pack(const float* fields, int32_t batch, int32_t h, int32_t w, const float* shift, const float* scale,
                 float* state, void* act, void* stream) {
     if (!fields || !shift || !scale || !state || batch < 1 || h < 1 || w < 1) return LBM_ERR_ARG;
-    const long long n = (long long)batch * h * w * 16;
-    pack_kernel<<<grid_for(n, 256), 256, 0, static_cast<cudaStream_t>(stream)>>>(
-        fields, batch, h, w, shift, scale, state, static_cast<__nv_bfloat16*>(act));
+    const long long hw = (long long)h * w;
+    pack_kernel<<<image_grid(hw, batch), 256, 0, static_cast<cudaStream_t>(stream)>>>(
+        fields, batch, hw, shift, scale, state, static_cast<__nv_bfloat16*>(act),
+        ((uintptr_t)state | (uintptr_t)act) % 16 == 0);
     return launch_status();
 }
 
 int lbm_nn_unpack(const float* state, int32_t batch, int32_t h, int32_t w, const float* shift, const float* scale,
                   float* fields, void* stream) {
     if (!state || !shift || !scale || !fields || batch < 1 || h < 1 || w < 1) return LBM_ERR_ARG;
-    const long long n = (long long)batch * h * w * 5;
-    unpack_kernel<<<grid_for(n, 256), 256, 0, static_cast<cudaStream_t>(stream)>>>(state, batch, h, w, shift, scale, fields);
+    const long long hw = (long long)h * w;
+    unpack_kernel<<<image_grid(hw, batch), 256, 0, static_cast<cudaStream_t>(stream)>>>(
+        state, batch, hw, shift, scale, fields, (uintptr_t)state % 16 == 0);
     return launch_status();
 }
 
