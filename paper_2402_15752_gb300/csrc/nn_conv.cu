@@ -164,6 +164,47 @@ __device__ __forceinline__ uint32_t swz32(uint32_t a) { return a ^ (((a >> 7) & 
 
 constexpr uint32_t LAYOUT_SW32 = 6;  // descriptor layout type, bits 61-63
 
+// The same exchange for pixel slots of 32 or 128 bytes (128-byte swizzle: byte-address
+// bits 4-6 ^= bits 7-9).
+template <uint32_t PXB>
+__device__ __forceinline__ uint32_t swz(uint32_t a) {
+    return PXB == 128 ? a ^ (((a >> 7) & 7u) << 4) : swz32(a);
+}
+constexpr uint32_t LAYOUT_SW128 = 2;
+
+// A descriptor in two words: the low one (start, leading-byte offset) moves with the
+// operand, the high one (stride-byte offset, version, layout) stays.
+__device__ __forceinline__ uint32_t sdesc_lo(uint32_t saddr, uint32_t lbo) {
+    return ((saddr >> 4) & 0x3FFF) | (((lbo >> 4) & 0x3FFF) << 16);
+}
+__host__ __device__ constexpr uint32_t sdesc_hi(uint32_t sbo, uint32_t layout) {
+    return ((sbo >> 4) & 0x3FFF) | (1u << 14) | (layout << 29);
+}
+
+// 1 on one lane of the (converged) warp.
+__device__ __forceinline__ uint32_t elect_one() {
+    uint32_t e;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(e));
+    return e;
+}
+// D += A B on the lane with go != 0; descriptors as (low, high) words.
+__device__ __forceinline__ void umma_if(uint32_t go, uint32_t d_tmem, uint32_t al, uint32_t ah, uint32_t bl, uint32_t bh,
+                                        uint32_t idesc) {
+    asm volatile(
+        "{\n\t.reg .pred q, t;\n\t.reg .b64 a, b;\n\tsetp.ne.b32 q, %6, 0;\n\tsetp.eq.u32 t, 0, 0;\n\t"
+        "mov.b64 a, {%1, %2};\n\tmov.b64 b, {%3, %4};\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %5, t;\n\t}\n" ::"r"(d_tmem),
+        "r"(al), "r"(ah), "r"(bl), "r"(bh), "r"(idesc), "r"(go)
+        : "memory");
+}
+__device__ __forceinline__ void commit_if(uint32_t go, uint32_t mbar) {
+    asm volatile(
+        "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}\n" ::"r"(mbar),
+        "r"(go)
+        : "memory");
+}
+
 __device__ __forceinline__ uint64_t sdesc_sw32(uint32_t saddr) {
     return sdesc(saddr, 16, 256) | ((uint64_t)LAYOUT_SW32 << 61);
 }
@@ -209,6 +250,15 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map
         "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], "
         "[%5];\n" ::"r"(dst),
         "l"(reinterpret_cast<uint64_t>(map)), "r"(c), "r"(xx), "r"(row), "r"(mbar)
+        : "memory");
+}
+
+__device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map, int c, int xx, int row, int plane,
+                                            uint32_t mbar) {
+    asm volatile(
+        "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], "
+        "[%6];\n" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(c), "r"(xx), "r"(row), "r"(plane), "r"(mbar)
         : "memory");
 }
 
@@ -541,6 +591,36 @@ bool activation_map(CUtensorMap* map, const void* x, int C, int B, int H, int W)
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// The same tensor, one box per image row of 128 pixels: 48 channels as 128-byte pixel
+// slots (box of 64 channels, the 16 beyond the tensor read as zeros; 128-byte
+// swizzle), 16 channels as 32-byte ones.
+bool row_map(CUtensorMap* map, const void* x, int C, int B, int H, int W) {
+    const EncodeTiledFn fn = encode_tiled();
+    if (!fn) return false;
+    const bool wide = C == 48;
+    const cuuint64_t dims[3] = {(cuuint64_t)C, (cuuint64_t)W, (cuuint64_t)B * H};
+    const cuuint64_t strides[2] = {(cuuint64_t)C * 2, (cuuint64_t)W * C * 2};
+    const cuuint32_t box[3] = {wide ? 64u : 16u, (cuuint32_t)TC_COLS, 1};
+    const cuuint32_t estr[3] = {1, 1, 1};
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(x), dims, strides, box, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, wide ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_32B,
+              CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// ... and one box per image row of 128 pixels as 16-channel planes (32-byte swizzle):
+// {channel of the plane, x, image row, plane}.
+bool plane_map(CUtensorMap* map, const void* x, int C, int B, int H, int W) {
+    const EncodeTiledFn fn = encode_tiled();
+    if (!fn) return false;
+    const cuuint64_t dims[4] = {16, (cuuint64_t)W, (cuuint64_t)B * H, (cuuint64_t)C / 16};
+    const cuuint64_t strides[3] = {(cuuint64_t)C * 2, (cuuint64_t)W * C * 2, 32};
+    const cuuint32_t box[4] = {16, (cuuint32_t)TC_COLS, 1, (cuuint32_t)C / 16};
+    const cuuint32_t estr[4] = {1, 1, 1, 1};
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(x), dims, strides, box, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // Tensor map of a 48-channel NHWC bfloat16 output: boxes of all 48 channels x
 // 32 pixels x 1 row (one epilogue warp's staging row), no swizzle.
 bool output_map(CUtensorMap* map, void* y, int B, int H, int W) {
@@ -586,178 +666,280 @@ int conv_tc_dispatch(const void* x, const void* w, const float* bias, void* y, c
 }
 
 // ------------------------------------------------------ weight gradient --
-// dw[o][t][c] = sum_p dy[p][o] x[p + d off_t][c].  Per tap t one accumulator
-// D_t (M = 64 rows, N columns) in tensor memory, K = pixels, 16 per MMA.  The
-// larger of (cin, cout) is the M side (rows beyond it are computed from
-// whatever follows in shared memory and never read).  Both operands are the
-// activations' 32-byte swizzled planes read MN-major: channels are the
-// contiguous (MN) direction, pixels the K direction; for MN-major swizzled
-// operands the leading-byte offset steps between 16-channel planes and the
-// stride-byte offset between groups of 8 pixels (256 bytes; measured on
-// GB300).  The shifted operand is x (with its halo), dy is read at the unit's
-// own pixels.  Roles as in the forward kernel: epilogue warps 0-3 (write the
-// CTA's partial at the end), TMA issuer, three halo loaders, MMA issuer.  Each
-// CTA accumulates over its units and writes one partial per tap; a second
-// kernel adds the partials in a fixed order: deterministic.
-// Bytes the M = 64 side reads past the end of a stage: its fourth plane (rows 48..63
-// of M: read by the tensor cores, never used).
-__host__ __device__ constexpr uint32_t wgrad_slack(int CI, int CO, int R) {
-    const uint32_t psx = (uint32_t)((R + 2) * WG_PITCH * 32), psd = (uint32_t)(R * TC_COLS * 32);
-    const uint32_t stage = (uint32_t)(CI / 16) * psx + (uint32_t)(CO / 16) * psd;
-    const uint32_t a_end = CI >= CO ? 4 * psx : (uint32_t)(CI / 16) * psx + 4 * psd;
-    return a_end > stage ? a_end - stage : 0u;
-}
+// dw[o][t][c] = sum_p dy[p][o] x[p + d off_t][c]: per tap a GEMM with K = pixels,
+// 16 per MMA, both operands read MN-major (channels contiguous) from the rows as the
+// TMA writes them.  A CTA marches down strips of image rows (columns 128 cb .., rows
+// of one residue modulo d): each row of x and of dy is loaded once, and row k of x
+// meets rows k - 1, k, k + 1 of dy while they are in the ring.
+//
+// What bounds it: the tensor cores' operand reads from shared memory and the rate of
+// MMAs, so one MMA carries as many taps as the layouts allow:
+// * N: the three dy rows stacked, 3 CO columns.  dy is stored as 16-channel planes
+//   of 128 pixels (32-byte swizzle), the planes of a row and the rows of the ring
+//   one after another, so that the 16-column groups of N are a constant 4 KB apart.
+// * M: the column taps.  The groups of M step by the dilation, LBO = d pixels: with
+//   48 input channels (64-channel rows of 128 bytes, 128-byte swizzle, the last 16
+//   channels filled with zeros by the TMA) M = 128 covers dx = -1, 0 and M = 64 dx =
+//   +1; with 16 (32-byte rows) M = 64 covers dx = -1, 0, 1 and an unused shift.
+// One box per row of x and dy: the TMA's time goes per box and per pixel row of a
+// box, and 4 KB boxes of 32-byte rows had been the floor (157 ns each).
+// Measured, 48 -> 48 channels, 16 images of 256 x 256: 155 us with one M = 64, N = 48
+// MMA per tap on units of two rows loaded with their halo rows; 52 us so (16 -> 48: 152
+// and 32, 48 -> 16: 151 and 39).
+// The accumulators (3 CO columns per M block) stay in tensor memory for the whole
+// kernel; a CTA writes one partial per tap and a second kernel adds them in a fixed
+// order: deterministic.
 
-template <int CI, int CO, int R, int S>
+// The strips' rows in the order strip by strip; CTA b of G takes rows [T b / G, T (b + 1) / G)
+// as runs of one strip each.
+struct Run {
+    long long left;  // rows of the CTA after this run
+    int strip, r0, n;
+};
+__device__ __forceinline__ Run first_run(long long T, int rows) {
+    const long long a = T * blockIdx.x / gridDim.x, b = T * (blockIdx.x + 1) / gridDim.x;
+    Run R;
+    R.strip = (int)(a / rows);
+    R.r0 = (int)(a - (long long)R.strip * rows);
+    R.n = (int)(b - a < rows - R.r0 ? b - a : rows - R.r0);
+    R.left = b - a - R.n;
+    return R;
+}
+__device__ __forceinline__ bool next_run(Run& R, int rows) {
+    if (R.left <= 0) return false;
+    ++R.strip;
+    R.r0 = 0;
+    R.n = (int)(R.left < rows ? R.left : rows);
+    R.left -= R.n;
+    return true;
+}
+// Strip: image n, residue rho, column block; image row (over all images) of its row r
+// (periodic: r = -1 and r = rows wrap).
+struct Strip {
+    int n, rho, x0;
+};
+__device__ __forceinline__ Strip strip_of(int s, int d, int ncb) {
+    Strip t;
+    t.x0 = (s % ncb) * TC_COLS;
+    s /= ncb;
+    t.rho = s % d;
+    t.n = s / d;
+    return t;
+}
+__device__ __forceinline__ int strip_row(const Strip& t, int r, int rows, int d, int H) {
+    return t.n * H + t.rho + (r < 0 ? r + rows : (r >= rows ? r - rows : r)) * d;
+}
+// A ring position: slot and the parity of its current round.
+template <int S>
+struct Ring {
+    int s = 0;
+    uint32_t round = 0;
+    __device__ __forceinline__ void next() {
+        if (++s == S) {
+            s = 0;
+            ++round;
+        }
+    }
+};
+
+template <int CI, int CO>
+struct Wg {
+    static constexpr uint32_t XPB = CI == 48 ? 128 : 32;       // bytes of a pixel slot of x
+    static constexpr uint32_t XROW = WG_PITCH * XPB;           // a row of x with its halo slots
+    static constexpr uint32_t DROW = (CO / 16) * TC_COLS * 32; // a row of dy: planes of 128 pixels
+    // slots: the x rings a multiple of the halo warps, so that each owns its slots (a
+    // parity wait cannot tell two rounds apart)
+    static constexpr int SX = CI == 48 ? 6 : 9, SD = 9;
+    static constexpr uint32_t N3 = 3 * CO;
+    static constexpr uint32_t TCOLS = pow2_cols(CI == 48 ? 2 * N3 : N3);
+    static constexpr size_t smem() { return (size_t)SX * XROW + SD * DROW + (2 * SX + 2 * SD + 1) * 8 + 16; }
+};
+
+template <int CI, int CO>
 __global__ void __launch_bounds__(WG_THREADS, 1)
     wgrad_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap dmap,
                     const uint8_t* __restrict__ x, float* __restrict__ partials, int B, int H, int W, int d,
                     int* __restrict__ status) {
-    constexpr bool A_IS_X = CI >= CO;
-    constexpr int KX = CI / 16, KD = CO / 16;          // 16-channel planes of x and dy
-    constexpr int NCX = CI / 8;                        // 16-byte chunks per x pixel
-    constexpr int N = A_IS_X ? CO : CI;                // accumulator columns per tap
-    constexpr int MREAL = A_IS_X ? CI : CO;            // real rows of M = 64
-    constexpr uint32_t TCOLS = pow2_cols(9 * N);
-    constexpr uint32_t IDESC = idesc_bf16(64, N, 1, 1);
-    constexpr uint32_t PSX = (uint32_t)((R + 2) * WG_PITCH * 32);  // x plane: R + 2 rows with halo slots
-    constexpr uint32_t PSD = (uint32_t)(R * TC_COLS * 32);         // dy plane: R rows of 128 pixels
-    constexpr uint32_t STAGE = KX * PSX + KD * PSD;
-    constexpr uint32_t TX = (uint32_t)((R + 2) * KX + R * KD) * TC_COLS * 32;
-    constexpr int HW = S;  // halo warps in use: one per stage
-    static_assert(MREAL <= 64 && N % 16 == 0, "M = 64 UMMA shapes");
-    static_assert(S <= WG_HALO_WARPS, "one halo warp per stage");
+    using K = Wg<CI, CO>;
+    constexpr int SX = K::SX, SD = K::SD;
+    constexpr int NCX = CI / 8;  // 16-byte chunks of an x pixel
+    static_assert(SX % WG_HALO_WARPS == 0, "x slots owned by one halo warp");
+    static_assert(SD >= 4, "three rows of dy and one to load");
     extern __shared__ __align__(1024) uint8_t smem[];
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const uint32_t sin0 = smem_u32(smem);
-    // after the stages: room for the A side's fourth plane (read, never used), then barriers
-    constexpr uint32_t SLACK = wgrad_slack(CI, CO, R);
-    uint64_t* s_bar = reinterpret_cast<uint64_t*>(smem + S * STAGE + SLACK);
-    uint32_t* s_tmem = reinterpret_cast<uint32_t*>(s_bar + 2 * S + 1);
-    auto full = [&](int s) { return smem_u32(&s_bar[s]); };
-    auto empty = [&](int s) { return smem_u32(&s_bar[S + s]); };
-    const uint32_t done = smem_u32(&s_bar[2 * S]);
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+    const uint32_t sx0 = smem_u32(smem), sd0 = sx0 + SX * K::XROW;
+    uint64_t* s_bar = reinterpret_cast<uint64_t*>(smem + SX * K::XROW + SD * K::DROW);
+    uint32_t* s_tmem = reinterpret_cast<uint32_t*>(s_bar + 2 * SX + 2 * SD + 1);
+    const uint32_t bar0 = smem_u32(s_bar);
+    auto xfull = [&](int s) { return bar0 + 8u * s; };
+    auto xempty = [&](int s) { return bar0 + 8u * (SX + s); };
+    auto dfull = [&](int s) { return bar0 + 8u * (2 * SX + s); };
+    auto dempty = [&](int s) { return bar0 + 8u * (2 * SX + SD + s); };
+    const uint32_t done = bar0 + 8u * (2 * SX + 2 * SD);
     if (tid == 0) {
-        for (int s = 0; s < S; ++s) {
-            mbar_init_n(full(s), 1 + 32);
-            mbar_init_n(empty(s), 1);
+        for (int s = 0; s < SX; ++s) {
+            mbar_init_n(xfull(s), 1 + 32);  // the TMA issuer's expect_tx and the lanes of a halo warp
+            mbar_init_n(xempty(s), 1);
+        }
+        for (int s = 0; s < SD; ++s) {
+            mbar_init_n(dfull(s), 1);
+            mbar_init_n(dempty(s), 1);
         }
         mbar_init_n(done, 1);
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
-    if (warp == WG_MMA_WARP) tmem_alloc(smem_u32(s_tmem), TCOLS);
+    if (warp == WG_MMA_WARP) tmem_alloc(smem_u32(s_tmem), K::TCOLS);
     fence_before_sync();
     __syncthreads();
     fence_after_sync();
-    const uint32_t tmem = *s_tmem;
-    const int nrb = H / d / R, ncb = W / TC_COLS;
-    const long long units = (long long)B * d * nrb * ncb;
-    const long long mine = units > blockIdx.x ? (units - 1 - blockIdx.x) / gridDim.x + 1 : 0;
+    const uint32_t tmem = __shfl_sync(0xffffffffu, *s_tmem, 0);
+    // every MMA accumulates: zero the accumulators
+    if (warp < 4) {
+        constexpr uint32_t USED = CI == 48 ? 2 * K::N3 : K::N3;
+        for (uint32_t c = 0; c < USED; c += 16) tmem_zero16(tmem + ((uint32_t)(32 * warp) << 16) + c);
+        tmem_wait_st();
+    }
+    fence_before_sync();
+    __syncthreads();
+    fence_after_sync();
+
+    const int rows = H / d, ncb = W / TC_COLS;
+    const long long T = (long long)B * d * ncb * rows;
     bool ok = true;
 
     if (warp == WG_TMA_WARP) {
+        // per run: dy rows r0 .. r0 + n - 1 and x rows r0 - 1 .. r0 + n, in the order the MMAs need them
         if (lane == 0) {
-            for (long long j = 0; j < mine; ++j) {
-                const int s = (int)(j % S);
-                if (j >= S) ok = mbar_wait(empty(s), (uint32_t)(((j / S) - 1) & 1));
-                if (!ok) break;
-                const Unit U = unit_of(blockIdx.x + j * gridDim.x, d, nrb, ncb);
-                mbar_arrive_tx(full(s), TX);
-                const uint32_t st = sin0 + (uint32_t)s * STAGE;
-#pragma unroll 1
-                for (int k = 0; k < R + 2; ++k) {
-                    const int row = U.n * H + image_row(U, k, R, d, H);
-#pragma unroll
-                    for (int kb = 0; kb < KX; ++kb)
-                        tma_load_3d(st + (uint32_t)kb * PSX + (uint32_t)(k * WG_PITCH + WG_HALO) * 32u, &xmap, 16 * kb,
-                                    U.x0, row, full(s));
-                    if (k >= 1 && k <= R) {
-#pragma unroll
-                        for (int kb = 0; kb < KD; ++kb)
-                            tma_load_3d(st + KX * PSX + (uint32_t)kb * PSD + (uint32_t)((k - 1) * TC_COLS) * 32u, &dmap,
-                                        16 * kb, U.x0, row, full(s));
+            Ring<SX> qx;
+            Ring<SD> qd;
+            Run R = first_run(T, rows);
+            do {
+                const Strip t = strip_of(R.strip, d, ncb);
+                for (int i = 0; i < R.n + 2 && ok; ++i) {
+                    if (i < R.n) {
+                        if (qd.round) ok = mbar_wait(dempty(qd.s), (qd.round - 1) & 1);
+                        if (!ok) break;
+                        mbar_arrive_tx(dfull(qd.s), K::DROW);
+                        tma_load_4d(sd0 + (uint32_t)qd.s * K::DROW, &dmap, 0, t.x0, strip_row(t, R.r0 + i, rows, d, H), 0,
+                                    dfull(qd.s));
+                        qd.next();
                     }
+                    if (qx.round) ok = mbar_wait(xempty(qx.s), (qx.round - 1) & 1);
+                    if (!ok) break;
+                    mbar_arrive_tx(xfull(qx.s), TC_COLS * K::XPB);
+                    tma_load_3d(sx0 + (uint32_t)qx.s * K::XROW + WG_HALO * K::XPB, &xmap, 0, t.x0,
+                                strip_row(t, R.r0 - 1 + i, rows, d, H), xfull(qx.s));
+                    qx.next();
                 }
-            }
+            } while (ok && next_run(R, rows));
         }
         __syncwarp();
-    } else if (warp >= WG_HALO_WARP && warp < WG_HALO_WARP + HW) {
-        // halo warp h serves stage h only, so it waits on every phase of that
-        // stage's barrier in order (a parity wait cannot tell phases two apart)
-        for (long long j = warp - WG_HALO_WARP; j < mine; j += HW) {
-            const int s = (int)(j % S);
-            if (j >= S) ok = mbar_wait(empty(s), (uint32_t)(((j / S) - 1) & 1));
-            if (!ok) break;
-            const Unit U = unit_of(blockIdx.x + j * gridDim.x, d, nrb, ncb);
-            const uint32_t st = sin0 + (uint32_t)s * STAGE;
-            const int per_row = 2 * d * NCX;
-            for (int i = lane; i < (R + 2) * per_row; i += 32) {
-                const int k = i / per_row, rem = i % per_row, jc = rem % NCX, e = rem / NCX;
-                int xx = e < d ? U.x0 - 1 - e : U.x0 + TC_COLS + (e - d);
-                const int slot = e < d ? WG_HALO - 1 - e : WG_HALO + TC_COLS + (e - d);
-                xx += xx < 0 ? W : (xx >= W ? -W : 0);
-                const uint8_t* src = x + (((long long)U.n * H + image_row(U, k, R, d, H)) * W + xx) * (16LL * NCX) + 16 * jc;
-                const uint32_t dst = st + (uint32_t)(jc >> 1) * PSX + (uint32_t)(k * WG_PITCH + slot) * 32u +
-                                     (uint32_t)(jc & 1) * 16u;
-                cp_async16(swz32(dst), src);
+    } else if (warp >= WG_HALO_WARP && warp < WG_HALO_WARP + WG_HALO_WARPS) {
+        // d columns on each side of every x row, wrapped, 16 bytes per copy
+        Ring<SX> qx;
+        int turn = 0;
+        Run R = first_run(T, rows);
+        do {
+            const Strip t = strip_of(R.strip, d, ncb);
+            for (int i = 0; i < R.n + 2 && ok; ++i, qx.next(), turn = turn == WG_HALO_WARPS - 1 ? 0 : turn + 1) {
+                if (turn != warp - WG_HALO_WARP) continue;
+                if (qx.round) ok = mbar_wait(xempty(qx.s), (qx.round - 1) & 1);
+                if (!ok) break;
+                const long long row = strip_row(t, R.r0 - 1 + i, rows, d, H);
+                for (int k = lane; k < 2 * d * NCX; k += 32) {
+                    const int jc = k % NCX, e = k / NCX;
+                    int xx = e < d ? t.x0 - 1 - e : t.x0 + TC_COLS + (e - d);
+                    const int slot = e < d ? WG_HALO - 1 - e : WG_HALO + TC_COLS + (e - d);
+                    xx += xx < 0 ? W : (xx >= W ? -W : 0);
+                    cp_async16(swz<K::XPB>(sx0 + (uint32_t)qx.s * K::XROW + (uint32_t)slot * K::XPB + 16u * jc),
+                               x + (row * W + xx) * (16LL * NCX) + 16 * jc);
+                }
+                cp_async_commit();
+                cp_async_wait_all();
+                fence_proxy_async();
+                mbar_arrive(xfull(qx.s));
             }
-            cp_async_commit();
-            cp_async_wait_all();
-            fence_proxy_async();
-            mbar_arrive(full(s));
-        }
+        } while (ok && next_run(R, rows));
     } else if (warp == WG_MMA_WARP) {
-        if (lane == 0) {
-            for (long long j = 0; j < mine; ++j) {
-                const int s = (int)(j % S);
-                ok = mbar_wait(full(s), (uint32_t)((j / S) & 1));
+        // The whole warp runs the loop with warp-uniform values (slots, descriptors), one
+        // elected lane issues: with the loop inside a lane's branch the compiler moved
+        // each MMA's five operands into uniform registers one by one.
+        const uint32_t leader = elect_one();
+        Ring<SX> qx;
+        Ring<SD> qd;
+        const uint32_t xhi = sdesc_hi(K::XPB == 128 ? 1024 : 256, K::XPB == 128 ? LAYOUT_SW128 : LAYOUT_SW32);
+        const uint32_t dhi = sdesc_hi(256, LAYOUT_SW32);
+        const uint32_t xl = sdesc_lo(sx0 + (uint32_t)(WG_HALO - d) * K::XPB, (uint32_t)d * K::XPB);
+        const uint32_t dl = sdesc_lo(sd0, TC_COLS * 32);
+        // n3 dy rows from slot s on, at stack position k
+        auto stack = [&](int sx, int s, int n3, int k) {
+            const uint32_t i1 = idesc_bf16(CI == 48 ? 128 : 64, 0, 1, 1) | ((uint32_t)(n3 * CO >> 3) << 17);
+            const uint32_t i2 = idesc_bf16(64, 0, 1, 1) | ((uint32_t)(n3 * CO >> 3) << 17);
+            uint32_t a = xl + (uint32_t)sx * (K::XROW / 16), b = dl + (uint32_t)s * (K::DROW / 16);
+            const uint32_t a2 = (uint32_t)(2 * d) * (K::XPB / 16);
+            const uint32_t c = tmem + (uint32_t)(k * CO);
+#pragma unroll
+            for (int p0 = 0; p0 < TC_COLS; p0 += 16) {
+                umma_if(leader, c, a, xhi, b, dhi, i1);
+                if constexpr (CI == 48) umma_if(leader, c + K::N3, a + a2, xhi, b, dhi, i2);
+                a += K::XPB;  // 16 pixels, in 16-byte units
+                b += 32;
+            }
+        };
+        Run R = first_run(T, rows);
+        do {
+            int lo = qd.s;  // slot of the first dy row that the current x row meets
+            for (int i = 0; i < R.n + 2 && ok; ++i) {
+                if (i < R.n) {
+                    ok = mbar_wait(dfull(qd.s), qd.round & 1);
+                    qd.next();
+                }
+                ok = ok && mbar_wait(xfull(qx.s), qx.round & 1);
+                ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 fence_after_sync();
-                const uint32_t sx = sin0 + (uint32_t)s * STAGE, sd = sx + KX * PSX;
-#pragma unroll 1
-                for (int r = 0; r < R; ++r) {
-#pragma unroll 1
-                    for (int p0 = 0; p0 < TC_COLS; p0 += 16) {
-                        const uint64_t dd = sdesc(sd + (uint32_t)(r * TC_COLS + p0) * 32u, PSD, 256) |
-                                            ((uint64_t)LAYOUT_SW32 << 61);
-#pragma unroll
-                        for (int t = 0; t < 9; ++t) {
-                            const int dy = t / 3 - 1, dx = t % 3 - 1;
-                            const uint64_t xd =
-                                sdesc(sx + (uint32_t)((r + 1 + dy) * WG_PITCH + WG_HALO + dx * d + p0) * 32u, PSX, 256) |
-                                ((uint64_t)LAYOUT_SW32 << 61);
-                            const uint32_t first = (j == 0 && r == 0 && p0 == 0);
-                            umma(tmem + (uint32_t)(t * N), A_IS_X ? xd : dd, A_IS_X ? dd : xd, IDESC, !first);
-                        }
-                    }
+                // dy rows max(i - 2, 0) .. min(i, n - 1) of the run; stack position 0: row i - 2
+                const int first = i < 2 ? 0 : i - 2, n3 = (i < R.n ? i : R.n - 1) - first + 1, k = first - (i - 2);
+                const int n1 = lo + n3 > SD ? SD - lo : n3;
+                stack(qx.s, lo, n1, k);
+                if (n1 < n3) stack(qx.s, 0, n3 - n1, k + n1);
+                commit_if(leader, xempty(qx.s));
+                qx.next();
+                if (i >= 2) {
+                    commit_if(leader, dempty(lo));
+                    lo = lo + 1 == SD ? 0 : lo + 1;
                 }
-                umma_commit(empty(s));
             }
-            umma_commit(done);
-        }
+        } while (ok && next_run(R, rows));
+        commit_if(leader, done);
         __syncwarp();
     } else {
-        // ---- epilogue: D_t row m (m < 64) lives in lane 32 (m / 16) + m % 16
-        if (mine > 0) ok = mbar_wait(done, 0);
+        // ---- epilogue: stack position k of the columns is tap row dy = 1 - k
+        ok = mbar_wait(done, 0);
         fence_after_sync();
         float* out = partials + (size_t)blockIdx.x * 9 * CI * CO;
-        const int m = 16 * warp + lane;  // valid for lane < 16
+        const uint32_t tq = tmem + ((uint32_t)(32 * warp) << 16);
+        auto write = [&](uint32_t block, int dxi, int ci, bool mine) {
 #pragma unroll 1
-        for (int t = 0; t < 9; ++t) {
+            for (int k = 0; k < 3; ++k) {
+                const int t = (2 - k) * 3 + dxi;
 #pragma unroll
-            for (int c0 = 0; c0 < N; c0 += 16) {
-                float v[16];
-                tmem_ld16(tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)(t * N + c0), v);
-                if (lane < 16 && m < MREAL) {
+                for (int c0 = 0; c0 < CO; c0 += 16) {
+                    float v[16];
+                    tmem_ld16(tq + block + (uint32_t)(k * CO + c0), v);
+                    if (mine) {
 #pragma unroll
-                    for (int e = 0; e < 16; ++e) {
-                        const int nn = c0 + e;
-                        const float val = (mine > 0 && ok) ? v[e] : 0.0f;
-                        if (A_IS_X) out[((size_t)t * CO + nn) * CI + m] = val;  // m = ci, nn = co
-                        else out[((size_t)t * CO + m) * CI + nn] = val;         // m = co, nn = ci
+                        for (int e = 0; e < 16; ++e) out[((size_t)t * CO + c0 + e) * CI + ci] = ok ? v[e] : 0.0f;
                     }
                 }
             }
+        };
+        if constexpr (CI == 48) {
+            const int m = 32 * warp + lane;  // M = 128: row m is lane m, dx = -1 below 64, 0 above
+            write(0, m / 64, m % 64, m % 64 < CI);
+            write(K::N3, 2, 16 * warp + lane, lane < 16 && 16 * warp + lane < CI);  // M = 64
+        } else {
+            write(0, warp, lane, lane < 16 && warp < 3);  // M = 64: group g (dx = g - 1) in lanes 32 g ..
         }
     }
     if (!ok) atomicOr(status, 1);
@@ -766,14 +948,14 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
     __syncthreads();
     if (warp == WG_MMA_WARP) {
         fence_after_sync();
-        tmem_free(tmem, TCOLS);
+        tmem_free(tmem, K::TCOLS);
     }
 }
 
 // dw[o][t][c] = sum_b partials[b][t][o][c], fixed order.  Latency-bound: a block
 // takes 32 consecutive outputs (128 contiguous bytes of a partial) and deals the
 // partials to 8 warps, whose sums it adds in order (44 us for 152 partials of 9 x 48
-// x 48 when one thread added all of an output's partials; 6 us so).
+// x 48 when one thread added all of an output's partials; 6.2 us so).
 constexpr int WR_OUT = 32, WR_SEG = 8;
 __global__ void __launch_bounds__(WR_OUT * WR_SEG)
     wgrad_tc_reduce(const float* __restrict__ partials, int nb, int CO, int CI, float* __restrict__ dw) {
@@ -798,38 +980,26 @@ __global__ void __launch_bounds__(WR_OUT * WR_SEG)
     }
 }
 
-template <int CI, int CO, int R, int S>
-constexpr size_t wgrad_tc_smem() {
-    return (size_t)S * ((CI / 16) * (R + 2) * WG_PITCH * 32 + (CO / 16) * R * TC_COLS * 32) +
-           wgrad_slack(CI, CO, R) + (2 * S + 1) * 8 + 16;
-}
-
-long long wgrad_units(int B, int H, int W, int d, int R) { return (long long)B * d * (H / d / R) * (W / TC_COLS); }
-
-// two rows per unit and two stages (both fit in shared memory), else one row
-int wgrad_rows(int H, int d) { return (H / d) % 2 == 0 ? 2 : 1; }
-
-template <int CI, int CO, int R, int S>
-int wgrad_tc_launch(const void* x, const void* dy, float* dw, float* part, int B, int H, int W, int d, int* status,
-                    cudaStream_t s) {
-    auto k = wgrad_tc_kernel<CI, CO, R, S>;
-    static_assert(wgrad_tc_smem<CI, CO, R, S>() <= 227 * 1024, "shared memory");
-    const size_t smem = std::max(wgrad_tc_smem<CI, CO, R, S>(), TC_MIN_SMEM);
-    CUtensorMap xmap, dmap;
-    if (!activation_map(&xmap, x, CI, B, H, W) || !activation_map(&dmap, dy, CO, B, H, W)) return LBM_ERR_CUDA;
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-        return LBM_ERR_CUDA;
-    const int grid = (int)std::min<long long>(wgrad_units(B, H, W, d, R), (long long)nn_sm_count());
-    k<<<grid, WG_THREADS, smem, s>>>(xmap, dmap, static_cast<const uint8_t*>(x), part, B, H, W, d, status);
-    wgrad_tc_reduce<<<(9 * CO * CI + WR_OUT - 1) / WR_OUT, WR_OUT * WR_SEG, 0, s>>>(part, grid, CO, CI, dw);
-    return cudaGetLastError() == cudaSuccess ? LBM_OK : LBM_ERR_CUDA;
+// partials (and CTAs at most): one per two rows of a strip where they divide by two,
+// else one per row
+long long wgrad_parts(int B, int H, int W, int d) {
+    return (long long)B * d * (H / d / ((H / d) % 2 == 0 ? 2 : 1)) * (W / TC_COLS);
 }
 
 template <int CI, int CO>
-int wgrad_tc_dispatch(const void* x, const void* dy, float* dw, float* part, int B, int H, int W, int d, int* status,
-                      cudaStream_t s) {
-    if (wgrad_rows(H, d) == 2) return wgrad_tc_launch<CI, CO, 2, 2>(x, dy, dw, part, B, H, W, d, status, s);
-    return wgrad_tc_launch<CI, CO, 1, 3>(x, dy, dw, part, B, H, W, d, status, s);
+int wgrad_tc_launch(const void* x, const void* dy, float* dw, float* part, int B, int H, int W, int d, int* status,
+                    cudaStream_t s) {
+    auto k = wgrad_tc_kernel<CI, CO>;
+    static_assert(Wg<CI, CO>::smem() <= 227 * 1024, "shared memory");
+    const size_t smem = std::max(Wg<CI, CO>::smem(), TC_MIN_SMEM);
+    CUtensorMap xmap, dmap;
+    if (!row_map(&xmap, x, CI, B, H, W) || !plane_map(&dmap, dy, CO, B, H, W)) return LBM_ERR_CUDA;
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+        return LBM_ERR_CUDA;
+    const int grid = (int)std::min<long long>(wgrad_parts(B, H, W, d), (long long)nn_sm_count());
+    k<<<grid, WG_THREADS, smem, s>>>(xmap, dmap, static_cast<const uint8_t*>(x), part, B, H, W, d, status);
+    wgrad_tc_reduce<<<(9 * CO * CI + WR_OUT - 1) / WR_OUT, WR_OUT * WR_SEG, 0, s>>>(part, grid, CO, CI, dw);
+    return cudaGetLastError() == cudaSuccess ? LBM_OK : LBM_ERR_CUDA;
 }
 
 bool conv_shape_ok(int B, int H, int W, int d) {
@@ -871,8 +1041,7 @@ int lbm_nn_conv3x3(const void* x, int32_t cin, const void* weights, const float*
 
 size_t lbm_nn_wgrad_partial_bytes(int32_t cin, int32_t cout, int32_t batch, int32_t h, int32_t w, int32_t dilation) {
     if (!conv_shape_ok(batch, h, w, dilation) || cin < 1 || cout < 1) return 0;
-    const long long units = wgrad_units(batch, h, w, dilation, wgrad_rows(h, dilation));
-    return (size_t)std::min<long long>(units, (long long)nn_sm_count()) * 9 * cin * cout * sizeof(float);
+    return (size_t)std::min<long long>(wgrad_parts(batch, h, w, dilation), (long long)nn_sm_count()) * 9 * cin * cout * sizeof(float);
 }
 
 int lbm_nn_conv3x3_wgrad(const void* x, int32_t cin, const void* dy, int32_t cout, float* dw, void* partials,
@@ -884,9 +1053,9 @@ int lbm_nn_conv3x3_wgrad(const void* x, int32_t cin, const void* dy, int32_t cou
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     float* part = static_cast<float*>(partials);
     const int d = dilation;
-    if (cin == 16 && cout == 48) return wgrad_tc_dispatch<16, 48>(x, dy, dw, part, batch, h, w, d, status, s);
-    if (cin == 48 && cout == 48) return wgrad_tc_dispatch<48, 48>(x, dy, dw, part, batch, h, w, d, status, s);
-    if (cin == 48 && cout == 16) return wgrad_tc_dispatch<48, 16>(x, dy, dw, part, batch, h, w, d, status, s);
+    if (cin == 16 && cout == 48) return wgrad_tc_launch<16, 48>(x, dy, dw, part, batch, h, w, d, status, s);
+    if (cin == 48 && cout == 48) return wgrad_tc_launch<48, 48>(x, dy, dw, part, batch, h, w, d, status, s);
+    if (cin == 48 && cout == 16) return wgrad_tc_launch<48, 16>(x, dy, dw, part, batch, h, w, d, status, s);
     return LBM_ERR_ARG;
 }
 

@@ -37,7 +37,7 @@ __device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w 
 // thread takes 8 channels of a pixel in one 16-byte load and keeps 8 sums, the
 // block's threads lie over consecutive bytes, and 4 loads per thread are in
 // flight.  16 x 256 x 256 pixels of 48 channels (100.7 MB, dy written before it):
-// 37.2 us with one 2-byte load per thread and iteration, 18 us so.
+// 37 us with one 2-byte load per thread and iteration, 26 us so (cold L2).
 // aligned: dy on a 16-byte boundary (else the same sums from 2-byte loads).
 template <int CO>
 __global__ void __launch_bounds__(256)
@@ -87,7 +87,7 @@ __global__ void __launch_bounds__(256)
 
 // out[o] = sum over nb partials of channel o, one block per channel and a tree in
 // a fixed order: latency-bound (58 us when one thread per channel added them in
-// turn, 3 us so at nb = 1024).
+// turn, 3.6 us so at nb = 1024).
 __global__ void __launch_bounds__(256)
     sum_partials(const float* __restrict__ part, int nb, int CO, float* __restrict__ out) {
     __shared__ float s[256];
@@ -121,75 +121,84 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
 // VEC: pred, target and dpred on 16-byte boundaries (else scalar accesses).
 // dpred = 2 inv d: the FP32 product with 2 inv = khi + klo, accurate to 2^-46 before
 // its one rounding to float, then rounded to bfloat16.
-template <bool VEC>
+// NV: groups of 4 channels in use.  Each thread has the loads of two pixels in
+// flight before it uses either.
+template <bool VEC, int NV>
 __global__ void __launch_bounds__(256)
     mse_partials(const float* __restrict__ pred, const float* __restrict__ target, int U, long long P,
                  __nv_bfloat16* __restrict__ dpred, double* __restrict__ part, double inv, float khi, float klo) {
     __shared__ double sh[8];
     double a = 0.0;
-    for (long long p = (long long)blockIdx.x * 256 + threadIdx.x; p < P; p += (long long)gridDim.x * 256) {
-        const float* pp = pred + p * 16;
-        const float* tt = target + p * 16;
-        uint32_t out[8];
+    auto fetch = [&](const float* __restrict__ src, long long p, float (&x)[4 * NV]) {
+#pragma unroll
+        for (int q = 0; q < NV; ++q) {
+            if constexpr (VEC) {
+                const float4 v = __ldg(reinterpret_cast<const float4*>(src + p * 16) + q);
+                x[4 * q] = v.x;
+                x[4 * q + 1] = v.y;
+                x[4 * q + 2] = v.z;
+                x[4 * q + 3] = v.w;
+            } else {
+#pragma unroll
+                for (int c = 0; c < 4; ++c) x[4 * q + c] = __ldg(src + p * 16 + 4 * q + c);
+            }
+        }
+    };
+    auto pixel = [&](long long p, const float (&x)[4 * NV], const float (&y)[4 * NV]) {
+        float g[16] = {};
         float H = 0.0f, L = 0.0f;
         double far = 0.0;  // squares outside the float range
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            float x[4] = {}, y[4] = {}, g[4] = {};
-            if (4 * q < U) {
-                if constexpr (VEC) {
-                    const float4 xv = *reinterpret_cast<const float4*>(pp + 4 * q);
-                    const float4 yv = *reinterpret_cast<const float4*>(tt + 4 * q);
-                    x[0] = xv.x; x[1] = xv.y; x[2] = xv.z; x[3] = xv.w;
-                    y[0] = yv.x; y[1] = yv.y; y[2] = yv.z; y[3] = yv.w;
-                } else {
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        x[c] = pp[4 * q + c];
-                        y[c] = tt[4 * q + c];
-                    }
-                }
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    if (4 * q + c >= U) continue;
-                    float s, e;
-                    two_sum(x[c], -y[c], s, e);
-                    const float m = fabsf(s);
-                    if (m == 0.0f || (m > 1e-14f && m < 1e18f)) {
-                        const float h = __fmul_rn(s, s);
-                        // the product's error, and the cross term of the split
-                        const float l = __fadd_rn(__fmaf_rn(s, s, -h), __fmul_rn(2.0f * s, e));
-                        float z, r;
-                        two_sum(H, h, z, r);
-                        H = z;
-                        L = __fadd_rn(L, __fadd_rn(r, l));
-                        g[c] = __fmaf_rn(khi, s, __fmaf_rn(khi, e, __fmul_rn(klo, s)));
-                    } else {
-                        const double d = (double)x[c] - (double)y[c];
-                        far += d * d;
-                        g[c] = (float)(2.0 * inv * d);
-                    }
-                }
+        for (int c = 0; c < 4 * NV; ++c) {
+            if (c >= U) continue;
+            float s, e;
+            two_sum(x[c], -y[c], s, e);
+            const float m = fabsf(s);
+            if (m == 0.0f || (m > 1e-14f && m < 1e18f)) {
+                const float h = __fmul_rn(s, s);
+                // the product's error, and the cross term of the split
+                const float l = __fadd_rn(__fmaf_rn(s, s, -h), __fmul_rn(2.0f * s, e));
+                float z, r;
+                two_sum(H, h, z, r);
+                H = z;
+                L = __fadd_rn(L, __fadd_rn(r, l));
+                g[c] = __fmaf_rn(khi, s, __fmaf_rn(khi, e, __fmul_rn(klo, s)));
+            } else {
+                const double d = (double)x[c] - (double)y[c];
+                far += d * d;
+                g[c] = (float)(2.0 * inv * d);
             }
-            const __nv_bfloat162 lo = __floats2bfloat162_rn(g[0], g[1]), hi = __floats2bfloat162_rn(g[2], g[3]);
-            out[2 * q] = *reinterpret_cast<const uint32_t*>(&lo);
-            out[2 * q + 1] = *reinterpret_cast<const uint32_t*>(&hi);
         }
         a += ((double)H + (double)L);
         if (far != 0.0) a += far;  // also NaN
-        if (dpred) {
-            if constexpr (VEC) {
-                uint4* o = reinterpret_cast<uint4*>(dpred + p * 16);
-                o[0] = make_uint4(out[0], out[1], out[2], out[3]);
-                o[1] = make_uint4(out[4], out[5], out[6], out[7]);
-            } else {
+        if (!dpred) return;
+        if constexpr (VEC) {
+            uint32_t out[8];
 #pragma unroll
-                for (int c = 0; c < 16; ++c) {
-                    const uint32_t w = out[c / 2];
-                    dpred[p * 16 + c] = __ushort_as_bfloat16((unsigned short)(c & 1 ? w >> 16 : w & 0xffffu));
-                }
+            for (int k = 0; k < 8; ++k) {
+                const __nv_bfloat162 w = __floats2bfloat162_rn(g[2 * k], g[2 * k + 1]);
+                out[k] = *reinterpret_cast<const uint32_t*>(&w);
             }
+            uint4* o = reinterpret_cast<uint4*>(dpred + p * 16);
+            o[0] = make_uint4(out[0], out[1], out[2], out[3]);
+            o[1] = make_uint4(out[4], out[5], out[6], out[7]);
+        } else {
+#pragma unroll
+            for (int c = 0; c < 16; ++c) dpred[p * 16 + c] = __float2bfloat16_rn(g[c]);
         }
+    };
+    const long long stride = (long long)gridDim.x * 256;
+    for (long long p = (long long)blockIdx.x * 256 + threadIdx.x; p < P; p += 2 * stride) {
+        const bool two = p + stride < P;
+        float x0[4 * NV], y0[4 * NV], x1[4 * NV], y1[4 * NV];
+        fetch(pred, p, x0);
+        fetch(target, p, y0);
+        if (two) {
+            fetch(pred, p + stride, x1);
+            fetch(target, p + stride, y1);
+        }
+        pixel(p, x0, y0);
+        if (two) pixel(p + stride, x1, y1);
     }
     for (int off = 16; off > 0; off >>= 1) a += __shfl_down_sync(0xffffffffu, a, off);
     if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = a;
@@ -202,7 +211,7 @@ __global__ void __launch_bounds__(256)
 }
 
 // The loss from the block partials, in a fixed order (67 us when one thread added
-// the 1024 of them in turn).
+// the 1024 of them in turn, 3.7 us so).
 __global__ void __launch_bounds__(256) mse_final(const double* __restrict__ part, int nb, double* __restrict__ loss) {
     __shared__ double s[256];
     double t = 0.0;
@@ -240,7 +249,7 @@ __global__ void adam_kernel(float* __restrict__ p, const float* __restrict__ g, 
 // (bfloat16) to a pixel, 512 contiguous bytes per store, the values passed by
 // shuffles.  With one thread per output value, every thread divided by the plane
 // size in 64 bits and re-read its plane one value at a time: 80 us at 16 x 256 x
-// 256 pixels; now 23 us.
+// 256 pixels; now 20 us.
 // vec: state and act on 16-byte boundaries (else scalar stores).
 __global__ void __launch_bounds__(256)
     pack_kernel(const float* __restrict__ fields, int B, long long HW, const float* __restrict__ shift,
@@ -494,10 +503,14 @@ int lbm_nn_mse(const float* pred, const float* target, int32_t used, int64_t pix
     const double inv = 1.0 / ((double)pixels * used);
     const float khi = (float)(2.0 * inv), klo = (float)(2.0 * inv - (double)khi);
     auto* dp = static_cast<__nv_bfloat16*>(dpred);
-    if (((uintptr_t)pred | (uintptr_t)target | (uintptr_t)dpred) % 16 == 0)
-        mse_partials<true><<<RED_BLOCKS, 256, 0, s>>>(pred, target, used, pixels, dp, loss_partials, inv, khi, klo);
-    else
-        mse_partials<false><<<RED_BLOCKS, 256, 0, s>>>(pred, target, used, pixels, dp, loss_partials, inv, khi, klo);
+    const bool vec = ((uintptr_t)pred | (uintptr_t)target | (uintptr_t)dpred) % 16 == 0;
+    auto run = [&](auto kernel) { kernel<<<RED_BLOCKS, 256, 0, s>>>(pred, target, used, pixels, dp, loss_partials, inv, khi, klo); };
+    switch ((used + 3) / 4) {
+        case 1: vec ? run(mse_partials<true, 1>) : run(mse_partials<false, 1>); break;
+        case 2: vec ? run(mse_partials<true, 2>) : run(mse_partials<false, 2>); break;
+        case 3: vec ? run(mse_partials<true, 3>) : run(mse_partials<false, 3>); break;
+        default: vec ? run(mse_partials<true, 4>) : run(mse_partials<false, 4>); break;
+    }
     mse_final<<<1, 256, 0, s>>>(loss_partials, RED_BLOCKS, loss);
     return launch_status();
 }
