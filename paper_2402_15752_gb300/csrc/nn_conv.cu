@@ -9,24 +9,22 @@
 // the 128 pixels of a row shifted by a tap (dy, dx) are the same layout at
 // another start address: a tap costs a descriptor, not a copy.  Activation
 // rows arrive by TMA (cp.async.bulk.tensor) in that layout; the periodic halo
-// columns of a unit by cp.async.
+// columns by cp.async.
 //
-// Descriptor fields (measured on GB300 with probe kernels against host
-// products): for no-swizzle K-major and MN-major operands the leading-byte
-// offset steps along K and the stride-byte offset along M/N; for 32-byte
-// swizzled MN-major operands the leading-byte offset steps between 16-element
-// MN groups and the stride-byte offset between 8-row K groups.  The swizzle
-// acts on absolute shared-memory address bits.  With M = 128 row m of the
-// accumulator is TMEM lane m; with M = 64, rows 16q .. 16q + 15 are lanes
-// 32q .. 32q + 15.  One thread issues a tcgen05.mma only about every 90 cycles,
-// so small-N MMAs need more than one issuing warp to keep the tensor cores busy.
+// Descriptor fields (measured on GB300 against host products): for swizzled K-major
+// operands the stride-byte offset steps between 8-row groups; for swizzled MN-major
+// operands the leading-byte offset steps between MN groups (of the swizzle's width)
+// and the stride-byte offset between 8-row K groups.  The swizzle acts on absolute
+// shared-memory address bits, so an operand may start at any pixel.  With M = 128 row
+// m of the accumulator is TMEM lane m; with M = 64, rows 16q .. 16q + 15 are lanes
+// 32q .. 32q + 15.
 //
-// Both kernels are persistent (one CTA per SM) over work units of R image rows
-// x 128 columns; with dilation d the rows of a unit are d apart, so its input
-// is R + 2 rows by 128 + 2d columns.  Warps have fixed roles (TMA issuer, halo
-// loaders, MMA issuers, epilogue) and hand off through mbarriers; every wait is
-// bounded: one that gives up sets bit 0 of *status and the CTA frees its tensor
-// memory and returns.
+// Both kernels are persistent (one CTA per SM) and march down strips of image rows:
+// 128 columns of the rows of one residue modulo the dilation d, so that each row of
+// the input is loaded once per strip and used by the three output rows it touches.
+// Warps have fixed roles (TMA issuer, halo loaders, MMA issuer, epilogue) and hand off
+// through mbarriers; every wait is bounded: one that gives up sets bit 0 of *status and
+// the CTA frees its tensor memory and returns.
 #include "lbm.h"
 #include "lbm_nn.h"
 #include "nn_internal.h"
@@ -49,33 +47,12 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
-// Shared-memory matrix descriptor, no swizzle: start, leading-byte offset
-// (along K), stride-byte offset (along M/N), all in 16-byte units; bit 46 is
-// the descriptor version of sm_100-class tensor cores.
-__device__ __forceinline__ uint64_t sdesc(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
-    return (uint64_t)((saddr >> 4) & 0x3FFF) | ((uint64_t)((lbo >> 4) & 0x3FFF) << 16) |
-           ((uint64_t)((sbo >> 4) & 0x3FFF) << 32) | ((uint64_t)1 << 46);
-}
-
 // Instruction descriptor of kind::f16: D FP32 (bits 4-5 = 1), A and B bfloat16
 // (bits 7-9, 10-12 = 1), A / B MN-major (bits 15 / 16), N >> 3 (bits 17-22),
 // M >> 4 (bits 24-28).
 constexpr uint32_t idesc_bf16(int M, int N, int a_mn, int b_mn) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)a_mn << 15) | ((uint32_t)b_mn << 16) |
            ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
-}
-
-__device__ __forceinline__ void umma(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
-        "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-
-__device__ __forceinline__ void umma_commit(uint32_t mbar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(mbar)
-                 : "memory");
 }
 
 __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity) {
@@ -136,22 +113,6 @@ __host__ __device__ constexpr uint32_t pow2_cols(uint32_t n) {
     return n <= 32 ? 32 : (n <= 64 ? 64 : (n <= 128 ? 128 : (n <= 256 ? 256 : 512)));
 }
 
-// A work unit: image n, residue rho of the rows modulo d, row block rb (rows
-// rho + (rb R + r) d, r < R), column block cb (columns 128 cb ..).
-struct Unit {
-    int n, rho, rb, x0;
-};
-__device__ __forceinline__ Unit unit_of(long long u, int d, int nrb, int ncb) {
-    Unit U;
-    U.x0 = (int)(u % ncb) * TC_COLS;
-    u /= ncb;
-    U.rb = (int)(u % nrb);
-    u /= nrb;
-    U.rho = (int)(u % d);
-    U.n = (int)(u / d);
-    return U;
-}
-
 // ------------------------------------------------------------ forward --
 // Operand layout of the forward kernel: 32-byte swizzled, K-major.  A row
 // (pixel, or weight row) is 16 channels = 32 bytes; groups of 8 rows are
@@ -172,8 +133,10 @@ __device__ __forceinline__ uint32_t swz(uint32_t a) {
 }
 constexpr uint32_t LAYOUT_SW128 = 2;
 
-// A descriptor in two words: the low one (start, leading-byte offset) moves with the
-// operand, the high one (stride-byte offset, version, layout) stays.
+// Shared-memory matrix descriptor in two words: the low one (start, leading-byte
+// offset, in 16-byte units) moves with the operand, the high one (stride-byte offset,
+// bit 46: the descriptor version of sm_100-class tensor cores, bits 61-63: the layout)
+// stays.
 __device__ __forceinline__ uint32_t sdesc_lo(uint32_t saddr, uint32_t lbo) {
     return ((saddr >> 4) & 0x3FFF) | (((lbo >> 4) & 0x3FFF) << 16);
 }
@@ -205,31 +168,20 @@ __device__ __forceinline__ void commit_if(uint32_t go, uint32_t mbar) {
         : "memory");
 }
 
-__device__ __forceinline__ uint64_t sdesc_sw32(uint32_t saddr) {
-    return sdesc(saddr, 16, 256) | ((uint64_t)LAYOUT_SW32 << 61);
-}
-
-// Roles of the forward kernel (warp index): 0-7 epilogue (warp w reads TMEM
-// lane quarter w % 4, output rows r = w / 4 mod 2), 8 the TMA issuer (lane 0),
-// 9-11 halo loaders (warp 9 + h loads the halos of stages q = h mod 3, so three
-// stages' halo copies are in flight at once), 12-13 the MMA issuers (lane 0;
-// warp 12 + p takes the units j = p mod 2 into accumulator buffer p: one thread
-// issues a tcgen05.mma only every ~90 cycles on GB300, two reach the tensor
-// cores' rate for these N <= 144 shapes (measured)); warp 12 owns the tensor memory.
+// Roles of the forward kernel (warp index): 0-7 epilogue (warp w reads TMEM lane
+// quarter w % 4 of the output rows g = w / 4 mod 2), 8 the TMA issuer (lane 0), 9-12
+// halo loaders (warp 9 + h the rows q = h mod 4), 13 the MMA issuer, which also owns
+// the tensor memory.
 constexpr int FW_EPI_WARPS = 8;
-constexpr int FW_TMA_WARP = 8, FW_HALO_WARP = 9, FW_HALO_WARPS = 3, FW_MMA_WARP = 12, FW_MMA_WARPS = 2;
+constexpr int FW_TMA_WARP = 8, FW_HALO_WARP = 9, FW_HALO_WARPS = 4, FW_MMA_WARP = 13;
 constexpr int FW_THREADS = 32 * 14;
 // Roles of the weight-gradient kernel: 0-3 epilogue, 4 TMA, 5-7 halo, 8 MMA.
 constexpr int WG_TMA_WARP = 4, WG_HALO_WARP = 5, WG_HALO_WARPS = 3, WG_MMA_WARP = 8;
 constexpr int WG_THREADS = 32 * 9;
-// A row of a stage plane: HALO halo slots, the 128 pixels of the unit, HALO
-// halo slots (dilation <= HALO, 4 or 8); the unit's first pixel sits 32 HALO
-// bytes into the row (128-byte aligned, as the TMA wants).  The weight-gradient
-// kernel uses 8.
-constexpr int WG_HALO = 8, WG_PITCH = TC_COLS + 2 * WG_HALO;
-// Output staging of the forward kernel: per epilogue warp one row of its 32
-// pixels x 48 bfloat16 channels (3 KB), written to global memory by a TMA store.
-constexpr uint32_t FW_STG = 32 * 48 * 2;
+// A row in shared memory: HALO halo slots, the 128 pixels of the strip, HALO halo slots
+// (dilation <= HALO); the first pixel sits HALO slots into the row, on a 1024-byte (48
+// channels) or 256-byte (16) boundary, where the swizzle's pattern starts.
+constexpr int HALO = 8, PITCH = TC_COLS + 2 * HALO;
 
 __device__ __forceinline__ void mbar_init_n(uint32_t mbar, uint32_t n) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(mbar), "r"(n) : "memory");
@@ -289,407 +241,6 @@ __device__ __forceinline__ void tmem_zero16(uint32_t taddr) {
 }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory"); }
 
-__device__ __forceinline__ int image_row(const Unit& U, int k, int R, int d, int H) {
-    int yy = U.rho + (U.rb * R + k - 1) * d;
-    return yy + (yy < 0 ? H : (yy >= H ? -H : 0));
-}
-
-// The three row taps (dy) share the A operand: for input row k of a unit, one
-// MMA multiplies the shifted row (dx) by the weights of all dy stacked along N
-// (rows ordered dy = +1, 0, -1), producing the contributions of that input row
-// to output rows k - 2, k - 1, k (those of the unit) in adjacent 48-column
-// blocks of tensor memory.  Output row i of a unit owns columns
-// [CO i, CO (i + 1)) of its buffer, so the three contributions to one output
-// row (from input rows i, i + 1, i + 2) accumulate on the same columns.  Half
-// the MMAs of one tap per MMA, each re-reading the 4 KB A tile for only 48 outputs.
-// Every MMA accumulates: the epilogue zeroes a buffer after reading it.
-template <int CI, int CO, int EPI, int R, int S, int HALO>
-__global__ void __launch_bounds__(FW_THREADS, 1)
-    conv_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap ymap,
-                   const uint8_t* __restrict__ x,
-                   const __nv_bfloat16* __restrict__ w, const float* __restrict__ bias, void* __restrict__ y,
-                   const float* __restrict__ res, const uint8_t* __restrict__ mask, int B, int H, int W, int d,
-                   int* __restrict__ status) {
-    static_assert(CI % 16 == 0 && CO % 16 == 0 && 3 * CO <= 256, "bfloat16 UMMA shapes");
-    constexpr int KB = CI / 16;                         // 16-channel planes of the input, K blocks per tap
-    constexpr int NC = CI / 8;                          // 16-byte chunks per input pixel
-    constexpr uint32_t WBYTES = 9u * CI * CO * 2u;
-    constexpr uint32_t ACC = (uint32_t)R * CO;          // TMEM columns of one unit
-    constexpr uint32_t TCOLS = pow2_cols(2 * ACC);
-    // a pipeline stage holds one 16-channel plane of a unit: (R + 2) rows of
-    // PITCH pixel slots, 32 bytes each (a multiple of 256 bytes)
-    constexpr int PITCH = TC_COLS + 2 * HALO;
-    constexpr uint32_t STAGE = (uint32_t)((R + 2) * PITCH * 32);
-    constexpr bool STAGED = CO == 48;                   // bfloat16 output through TMA stores
-    constexpr uint32_t STG = STAGED ? FW_EPI_WARPS * FW_STG : 0u;
-    constexpr uint32_t TX = (uint32_t)((R + 2) * TC_COLS * 32);  // TMA bytes per stage
-    // halo warp h serves the stages s = h mod 3 only, and MMA warp p the stages
-    // of the units j = p mod 2, so each waits on every phase of its stages'
-    // barriers in order (a parity wait cannot tell phases two apart)
-    static_assert(S % FW_HALO_WARPS == 0 && S % (2 * KB) == 0, "stages owned by one halo and one MMA warp");
-    extern __shared__ __align__(1024) uint8_t smem[];
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    // [stages][output staging][weights][bias][barriers: full S, empty S, tfull 2, tempty 2][tmem slot]
-    const uint32_t base = smem_u32(smem);
-    const uint32_t sin0 = base, sstg = base + S * STAGE, sw0 = sstg + STG;
-    float* s_bias = reinterpret_cast<float*>(smem + S * STAGE + STG + WBYTES);
-    uint64_t* s_bar = reinterpret_cast<uint64_t*>(s_bias + CO);
-    uint32_t* s_tmem = reinterpret_cast<uint32_t*>(s_bar + 2 * S + 4);
-    auto full = [&](int s) { return smem_u32(&s_bar[s]); };
-    auto empty = [&](int s) { return smem_u32(&s_bar[S + s]); };
-    auto tfull = [&](int b) { return smem_u32(&s_bar[2 * S + b]); };
-    auto tempty = [&](int b) { return smem_u32(&s_bar[2 * S + 2 + b]); };
-
-    // weights [co][t][ci] -> blocks (dx, 16-channel group) of 3 CO rows x 32
-    // bytes, swizzled; row bi CO + o of a block holds tap dy = 1 - bi
-    for (int i = tid; i < 9 * NC * CO; i += FW_THREADS) {
-        const int o = i % CO, rest = i / CO, j = rest % NC, tap = rest / NC;  // tap = 3 bi + dxi
-        const int bi = tap / 3, dxi = tap % 3, t = 3 * (2 - bi) + dxi;
-        const uint4 v = *reinterpret_cast<const uint4*>(w + ((size_t)o * 9 + t) * CI + 8 * j);
-        const uint32_t a = sw0 + (uint32_t)(((dxi * KB + (j >> 1)) * 3 + bi) * CO + o) * 32u + (uint32_t)(j & 1) * 16u;
-        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};\n" ::"r"(swz32(a)), "r"(v.x), "r"(v.y), "r"(v.z),
-                     "r"(v.w)
-                     : "memory");
-    }
-    for (int i = tid; i < CO; i += FW_THREADS) s_bias[i] = (EPI != LBM_NN_MASK && bias) ? bias[i] : 0.0f;
-    if (tid == 0) {
-        for (int s = 0; s < S; ++s) {
-            mbar_init_n(full(s), 1 + 32);  // the TMA issuer's expect_tx and the 32 lanes of one halo warp
-            mbar_init_n(empty(s), 1);
-        }
-        for (int b = 0; b < 2; ++b) {
-            mbar_init_n(tfull(b), 1);
-            mbar_init_n(tempty(b), 32 * FW_EPI_WARPS);
-        }
-        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-    }
-    if (warp == FW_MMA_WARP) tmem_alloc(smem_u32(s_tmem), TCOLS);
-    fence_proxy_async();  // the weights (generic stores) before the tensor cores read them
-    fence_before_sync();
-    __syncthreads();
-    fence_after_sync();
-    const uint32_t tmem = *s_tmem;
-    // the accumulators start at zero (every MMA accumulates)
-    if (warp < FW_EPI_WARPS) {
-        const uint32_t tq = tmem + ((uint32_t)(32 * (warp & 3)) << 16);
-        for (int r = warp >> 2; r < R; r += 2)
-            for (int b = 0; b < 2; ++b)
-#pragma unroll
-                for (int c0 = 0; c0 < CO; c0 += 16) tmem_zero16(tq + (uint32_t)(b * ACC + r * CO + c0));
-        tmem_wait_st();
-    }
-    fence_before_sync();
-    __syncthreads();
-    fence_after_sync();
-
-    const int nrb = H / d / R, ncb = W / TC_COLS;
-    const long long units = (long long)B * d * nrb * ncb;
-    const long long mine = units > blockIdx.x ? (units - 1 - blockIdx.x) / gridDim.x + 1 : 0;
-    bool ok = true;
-
-    if (warp == FW_TMA_WARP) {
-        // ---- TMA issuer: the unit's 128 columns of R + 2 rows, one box per row
-        if (lane == 0) {
-            for (long long q = 0; q < mine * KB; ++q) {
-                const int s = (int)(q % S), kb = (int)(q % KB);
-                if (q >= S) ok = mbar_wait(empty(s), (uint32_t)(((q / S) - 1) & 1));
-                if (!ok) break;
-                const Unit U = unit_of(blockIdx.x + (q / KB) * gridDim.x, d, nrb, ncb);
-                mbar_arrive_tx(full(s), TX);
-                const uint32_t st = sin0 + (uint32_t)s * STAGE;
-#pragma unroll 1
-                for (int k = 0; k < R + 2; ++k)
-                    tma_load_3d(st + (uint32_t)(k * PITCH + HALO) * 32u, &xmap, 16 * kb, U.x0,
-                                U.n * H + image_row(U, k, R, d, H), full(s));
-            }
-        }
-        __syncwarp();
-    } else if (warp >= FW_HALO_WARP && warp < FW_HALO_WARP + FW_HALO_WARPS) {
-        // ---- halo loaders: d columns on each side, wrapped, 16 bytes per copy
-        for (long long q = warp - FW_HALO_WARP; q < mine * KB; q += FW_HALO_WARPS) {
-            const int s = (int)(q % S), kb = (int)(q % KB);
-            if (q >= S) ok = mbar_wait(empty(s), (uint32_t)(((q / S) - 1) & 1));
-            if (!ok) break;
-            const Unit U = unit_of(blockIdx.x + (q / KB) * gridDim.x, d, nrb, ncb);
-            const uint32_t st = sin0 + (uint32_t)s * STAGE;
-            const int per_row = 2 * d * 2;  // 2d columns x two 16-byte halves of the plane
-            for (int i = lane; i < (R + 2) * per_row; i += 32) {
-                const int k = i / per_row, rem = i % per_row, h = rem & 1, e = rem >> 1;  // e < 2d
-                // e < d: left column x0 - 1 - e (slot HALO - 1 - e); else right column x0 + 128 + (e - d)
-                int xx = e < d ? U.x0 - 1 - e : U.x0 + TC_COLS + (e - d);
-                const int slot = e < d ? HALO - 1 - e : HALO + TC_COLS + (e - d);
-                xx += xx < 0 ? W : (xx >= W ? -W : 0);
-                const uint8_t* src = x + (((long long)U.n * H + image_row(U, k, R, d, H)) * W + xx) * (16LL * NC) +
-                                     32 * kb + 16 * h;
-                const uint32_t dst = st + (uint32_t)(k * PITCH + slot) * 32u + (uint32_t)h * 16u;
-                cp_async16(swz32(dst), src);
-            }
-            cp_async_commit();
-            cp_async_wait_all();
-            fence_proxy_async();
-            mbar_arrive(full(s));
-        }
-    } else if (warp >= FW_MMA_WARP) {
-        // ---- MMA issuers: per plane, per input row k, per column tap dx
-        if (lane == 0) {
-            for (long long j = warp - FW_MMA_WARP; j < mine && ok; j += FW_MMA_WARPS) {
-                const int b = (int)(j & 1);
-                if (j >= 2) ok = mbar_wait(tempty(b), (uint32_t)(((j >> 1) - 1) & 1));
-#pragma unroll 1
-                for (int kb = 0; kb < KB && ok; ++kb) {
-                    const long long q = j * KB + kb;
-                    const int s = (int)(q % S);
-                    ok = mbar_wait(full(s), (uint32_t)((q / S) & 1));
-                    if (!ok) break;
-                    fence_after_sync();
-                    const uint32_t sa = sin0 + (uint32_t)s * STAGE;
-#pragma unroll 1
-                    for (int k = 0; k < R + 2; ++k) {
-                        // output rows lo .. hi of the unit receive input row k (dy = k - 1 - i)
-                        const int lo = k - 2 > 0 ? k - 2 : 0, hi = k < R - 1 ? k : R - 1;
-                        const int n = (hi - lo + 1) * CO, bi = 2 - k + lo;
-                        const uint32_t idesc = idesc_bf16(128, n, 0, 0);
-                        const uint32_t dcol = tmem + (uint32_t)b * ACC + (uint32_t)(lo * CO);
-#pragma unroll
-                        for (int dxi = 0; dxi < 3; ++dxi) {
-                            const uint32_t aoff = (uint32_t)((k * PITCH + HALO + (dxi - 1) * d) * 32);
-                            umma(dcol, sdesc_sw32(sa + aoff),
-                                 sdesc_sw32(sw0 + (uint32_t)(((dxi * KB + kb) * 3 + bi) * CO) * 32u), idesc, 1u);
-                        }
-                    }
-                    umma_commit(empty(s));
-                }
-                if (ok) umma_commit(tfull(b));
-            }
-        }
-        __syncwarp();
-    } else {
-        // ---- epilogue: TMEM lane quarter warp % 4, pixel x0 + 32 (warp % 4) + lane,
-        // output rows r = warp / 4 (mod 2)
-        const int quarter = warp & 3;
-        const uint32_t stg = sstg + (uint32_t)warp * FW_STG;  // this warp's output staging row
-        for (long long j = 0; j < mine; ++j) {
-            const int b = (int)(j & 1);
-            ok = mbar_wait(tfull(b), (uint32_t)((j >> 1) & 1));
-            if (!ok) break;
-            fence_after_sync();
-            const Unit U = unit_of(blockIdx.x + j * gridDim.x, d, nrb, ncb);
-            const uint32_t tb = tmem + ((uint32_t)(32 * quarter) << 16) + (uint32_t)b * ACC;
-#pragma unroll 1
-            for (int r = warp >> 2; r < R; r += 2) {
-                const int yy = U.rho + (U.rb * R + r) * d;
-                const long long px = ((long long)U.n * H + yy) * W + U.x0 + 32 * quarter + lane;
-                if constexpr (CO == 48) {
-                    float v[48];
-                    tmem_ld48(tb + (uint32_t)(r * CO), v);
-                    uint32_t o[24];
-                    if constexpr (EPI == LBM_NN_RELU) {
-#pragma unroll
-                        for (int q = 0; q < 24; ++q)
-                            o[q] = pack_bf16x2(fmaxf(v[2 * q] + s_bias[2 * q], 0.0f),
-                                               fmaxf(v[2 * q + 1] + s_bias[2 * q + 1], 0.0f));
-                    } else {
-                        static_assert(EPI == LBM_NN_MASK || CO != 48, "48-channel epilogues: ReLU or mask");
-                        const uint4* mo = reinterpret_cast<const uint4*>(mask + px * CO * 2);
-#pragma unroll
-                        for (int q4 = 0; q4 < 6; ++q4) {
-                            const uint4 m4 = mo[q4];
-                            const uint32_t mk[4] = {m4.x, m4.y, m4.z, m4.w};
-#pragma unroll
-                            for (int e = 0; e < 4; ++e) {
-                                const int q = 4 * q4 + e;
-                                o[q] = pack_bf16x2(bf16_lo(mk[e]) > 0.0f ? v[2 * q] : 0.0f,
-                                                   bf16_hi(mk[e]) > 0.0f ? v[2 * q + 1] : 0.0f);
-                            }
-                        }
-                    }
-                    // the previous TMA store from this staging row has read it
-                    if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");
-                    __syncwarp();
-#pragma unroll
-                    for (int q4 = 0; q4 < 6; ++q4)
-                        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};\n" ::"r"(stg + (uint32_t)(lane * 96 + 16 * q4)),
-                                     "r"(o[4 * q4]), "r"(o[4 * q4 + 1]), "r"(o[4 * q4 + 2]), "r"(o[4 * q4 + 3])
-                                     : "memory");
-                    fence_proxy_async();  // the staging row (generic stores) before the TMA reads it
-                    __syncwarp();
-                    if (lane == 0) {
-                        asm volatile(
-                            "cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%1, %2, %3}], [%4];\n" ::"l"(
-                                reinterpret_cast<uint64_t>(&ymap)),
-                            "r"(0), "r"(U.x0 + 32 * quarter), "r"((int)(U.n * H + yy)), "r"(stg)
-                            : "memory");
-                        asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
-                    }
-                } else {
-                    static_assert(EPI == LBM_NN_RESIDUAL && CO == 16, "16-channel epilogue: residual");
-                    float v[16];
-                    tmem_ld16(tb + (uint32_t)(r * CO), v);
-                    const float4* ro = reinterpret_cast<const float4*>(res + px * CO);
-                    float4* yo = reinterpret_cast<float4*>(static_cast<float*>(y) + px * CO);
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const float4 a = ro[q];
-                        yo[q] = make_float4(a.x + v[4 * q] + s_bias[4 * q], a.y + v[4 * q + 1] + s_bias[4 * q + 1],
-                                            a.z + v[4 * q + 2] + s_bias[4 * q + 2], a.w + v[4 * q + 3] + s_bias[4 * q + 3]);
-                    }
-                }
-#pragma unroll
-                for (int c0 = 0; c0 < CO; c0 += 16) tmem_zero16(tb + (uint32_t)(r * CO + c0));
-            }
-            tmem_wait_st();
-            fence_before_sync();
-            mbar_arrive(tempty(b));
-        }
-        // every TMA store of this warp complete before the CTA (and its staging) goes away
-        if (STAGED && lane == 0) asm volatile("cp.async.bulk.wait_group 0;\n" ::: "memory");
-    }
-    if (!ok) atomicOr(status, 1);
-    cp_async_wait_all();
-    fence_before_sync();
-    __syncthreads();
-    if (warp == FW_MMA_WARP) {
-        fence_after_sync();
-        tmem_free(tmem, TCOLS);
-    }
-}
-
-template <int CI, int CO, int R, int S, int HALO>
-constexpr size_t conv_tc_smem() {
-    return (size_t)S * ((R + 2) * (TC_COLS + 2 * HALO) * 32) + (CO == 48 ? FW_EPI_WARPS * FW_STG : 0) +
-           9u * CI * CO * 2u + CO * 4 + (2 * S + 4) * 8 + 16;
-}
-
-// Tensor map of an NHWC bfloat16 activation: {channel, x, image row}, boxes of
-// 16 channels x 128 pixels x 1 row, 32-byte swizzle.
-using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeTiledFn encode_tiled() {
-    static EncodeTiledFn fn = nullptr;
-    if (!fn) {
-        void* p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
-                cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<EncodeTiledFn>(p);
-    }
-    return fn;
-}
-
-bool activation_map(CUtensorMap* map, const void* x, int C, int B, int H, int W) {
-    const EncodeTiledFn fn = encode_tiled();
-    if (!fn) return false;
-    const cuuint64_t dims[3] = {(cuuint64_t)C, (cuuint64_t)W, (cuuint64_t)B * H};
-    const cuuint64_t strides[2] = {(cuuint64_t)C * 2, (cuuint64_t)W * C * 2};
-    const cuuint32_t box[3] = {16, (cuuint32_t)TC_COLS, 1};
-    const cuuint32_t estr[3] = {1, 1, 1};
-    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(x), dims, strides, box, estr,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-// The same tensor, one box per image row of 128 pixels: 48 channels as 128-byte pixel
-// slots (box of 64 channels, the 16 beyond the tensor read as zeros; 128-byte
-// swizzle), 16 channels as 32-byte ones.
-bool row_map(CUtensorMap* map, const void* x, int C, int B, int H, int W) {
-    const EncodeTiledFn fn = encode_tiled();
-    if (!fn) return false;
-    const bool wide = C == 48;
-    const cuuint64_t dims[3] = {(cuuint64_t)C, (cuuint64_t)W, (cuuint64_t)B * H};
-    const cuuint64_t strides[2] = {(cuuint64_t)C * 2, (cuuint64_t)W * C * 2};
-    const cuuint32_t box[3] = {wide ? 64u : 16u, (cuuint32_t)TC_COLS, 1};
-    const cuuint32_t estr[3] = {1, 1, 1};
-    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(x), dims, strides, box, estr,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, wide ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_32B,
-              CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-// ... and one box per image row of 128 pixels as 16-channel planes (32-byte swizzle):
-// {channel of the plane, x, image row, plane}.
-bool plane_map(CUtensorMap* map, const void* x, int C, int B, int H, int W) {
-    const EncodeTiledFn fn = encode_tiled();
-    if (!fn) return false;
-    const cuuint64_t dims[4] = {16, (cuuint64_t)W, (cuuint64_t)B * H, (cuuint64_t)C / 16};
-    const cuuint64_t strides[3] = {(cuuint64_t)C * 2, (cuuint64_t)W * C * 2, 32};
-    const cuuint32_t box[4] = {16, (cuuint32_t)TC_COLS, 1, (cuuint32_t)C / 16};
-    const cuuint32_t estr[4] = {1, 1, 1, 1};
-    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(x), dims, strides, box, estr,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-// Tensor map of a 48-channel NHWC bfloat16 output: boxes of all 48 channels x
-// 32 pixels x 1 row (one epilogue warp's staging row), no swizzle.
-bool output_map(CUtensorMap* map, void* y, int B, int H, int W) {
-    const EncodeTiledFn fn = encode_tiled();
-    if (!fn) return false;
-    const cuuint64_t dims[3] = {48, (cuuint64_t)W, (cuuint64_t)B * H};
-    const cuuint64_t strides[2] = {96, (cuuint64_t)W * 96};
-    const cuuint32_t box[3] = {48, 32, 1};
-    const cuuint32_t estr[3] = {1, 1, 1};
-    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, y, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-              CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) ==
-           CUDA_SUCCESS;
-}
-
-template <int CI, int CO, int EPI, int R, int S, int HALO>
-int conv_tc_launch(const void* x, const void* w, const float* bias, void* y, const float* res, const void* mask, int B,
-                   int H, int W, int d, int* status, cudaStream_t s) {
-    auto k = conv_tc_kernel<CI, CO, EPI, R, S, HALO>;
-    const size_t smem = std::max(conv_tc_smem<CI, CO, R, S, HALO>(), TC_MIN_SMEM);
-    static_assert(conv_tc_smem<CI, CO, R, S, HALO>() <= 227 * 1024, "shared memory");
-    CUtensorMap map, ymap;
-    if (!activation_map(&map, x, CI, B, H, W)) return LBM_ERR_CUDA;
-    if (CO == 48 ? !output_map(&ymap, y, B, H, W) : !activation_map(&ymap, x, CI, B, H, W)) return LBM_ERR_CUDA;
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-        return LBM_ERR_CUDA;
-    const long long units = (long long)B * d * (H / d / R) * (W / TC_COLS);
-    const int grid = (int)std::min<long long>(units, (long long)nn_sm_count());
-    k<<<grid, FW_THREADS, smem, s>>>(map, ymap, static_cast<const uint8_t*>(x), static_cast<const __nv_bfloat16*>(w),
-                                     bias, y, res, static_cast<const uint8_t*>(mask), B, H, W, d, status);
-    return cudaGetLastError() == cudaSuccess ? LBM_OK : LBM_ERR_CUDA;
-}
-
-// Rows per unit, stages (one 16-channel plane of a unit each) and halo slots:
-// 4 rows, 6 stages, 4 halo slots for dilations up to 4 where the rows divide by
-// 4; else 2 rows, 6 stages, 8 slots where they divide by 2; else 1 row.
-template <int CI, int CO, int EPI>
-int conv_tc_dispatch(const void* x, const void* w, const float* bias, void* y, const float* res, const void* mask,
-                     int B, int H, int W, int d, int* status, cudaStream_t s) {
-    if ((H / d) % 4 == 0 && d <= 4)
-        return conv_tc_launch<CI, CO, EPI, 4, 6, 4>(x, w, bias, y, res, mask, B, H, W, d, status, s);
-    if ((H / d) % 2 == 0) return conv_tc_launch<CI, CO, EPI, 2, 6, 8>(x, w, bias, y, res, mask, B, H, W, d, status, s);
-    return conv_tc_launch<CI, CO, EPI, 1, 6, 8>(x, w, bias, y, res, mask, B, H, W, d, status, s);
-}
-
-// ------------------------------------------------------ weight gradient --
-// dw[o][t][c] = sum_p dy[p][o] x[p + d off_t][c]: per tap a GEMM with K = pixels,
-// 16 per MMA, both operands read MN-major (channels contiguous) from the rows as the
-// TMA writes them.  A CTA marches down strips of image rows (columns 128 cb .., rows
-// of one residue modulo d): each row of x and of dy is loaded once, and row k of x
-// meets rows k - 1, k, k + 1 of dy while they are in the ring.
-//
-// What bounds it: the tensor cores' operand reads from shared memory and the rate of
-// MMAs, so one MMA carries as many taps as the layouts allow:
-// * N: the three dy rows stacked, 3 CO columns.  dy is stored as 16-channel planes
-//   of 128 pixels (32-byte swizzle), the planes of a row and the rows of the ring
-//   one after another, so that the 16-column groups of N are a constant 4 KB apart.
-// * M: the column taps.  The groups of M step by the dilation, LBO = d pixels: with
-//   48 input channels (64-channel rows of 128 bytes, 128-byte swizzle, the last 16
-//   channels filled with zeros by the TMA) M = 128 covers dx = -1, 0 and M = 64 dx =
-//   +1; with 16 (32-byte rows) M = 64 covers dx = -1, 0, 1 and an unused shift.
-// One box per row of x and dy: the TMA's time goes per box and per pixel row of a
-// box, and 4 KB boxes of 32-byte rows had been the floor (157 ns each).
-// Measured, 48 -> 48 channels, 16 images of 256 x 256: 155 us with one M = 64, N = 48
-// MMA per tap on units of two rows loaded with their halo rows; 52 us so (16 -> 48: 152
-// and 32, 48 -> 16: 151 and 39).
-// The accumulators (3 CO columns per M block) stay in tensor memory for the whole
-// kernel; a CTA writes one partial per tap and a second kernel adds them in a fixed
-// order: deterministic.
-
 // The strips' rows in the order strip by strip; CTA b of G takes rows [T b / G, T (b + 1) / G)
 // as runs of one strip each.
 struct Run {
@@ -742,10 +293,407 @@ struct Ring {
     }
 };
 
+// One output row (128 pixels x CO channels) is a slot of CO columns of a TMEM ring.
+// Input row r of a strip meets the weights of its three row taps stacked along N (dy =
+// +1, 0, -1), whose products go to output rows r - 1, r, r + 1 in adjacent slots: N =
+// 3 CO, one MMA per 16 input channels and column tap (the shifted row is the same rows
+// of shared memory from another start).  Every MMA accumulates: the epilogue zeroes a
+// slot after reading it.
+//
+// Order of accumulation: an output takes its 16-channel groups one after another,
+// within a group the input rows r - 1, r, r + 1, within a row the column taps (the
+// order of a kernel that holds whole units of rows).  So group g of an input row is
+// issued 2 g rows after its first group, when group g - 1 of the next row has been.
+//
+// What bounds it: HBM (a row in and out per output row; the MMAs of a row take about
+// 0.35 us of the 0.55 us that its bytes take).  48 -> 48 channels, 16 images of 256 x
+// 256: units of 4 rows loaded with their 2 halo rows as 18 boxes of 4 KB took 54 us
+// (76 at dilation 8, units of 2 rows) and 66 us (77) with the mask epilogue, bound by
+// the TMA's time per box and pixel row; one box of 128-byte pixel slots per row,
+// loaded once: @F@.
+template <int CI, int CO>
+struct Fw {
+    static constexpr int KB = CI / 16;                         // 16-channel groups of the input
+    static constexpr uint32_t XPB = CI == 48 ? 128 : 32;       // bytes of a pixel slot
+    static constexpr uint32_t XROW = PITCH * XPB;
+    static constexpr int S = CI == 48 ? 8 : 16;                // rows in the ring: 2 KB - 1 in use, the rest in flight
+    static constexpr int NT = 10;                              // output slots: 2 KB + 1 open, the rest in the epilogue
+    static constexpr uint32_t WBYTES = 9u * CI * CO * 2u;
+    static constexpr uint32_t OUT = 32 * (CO == 48 ? 96 : 64); // a warp's 32 output pixels
+    static constexpr uint32_t TCOLS = pow2_cols(NT * CO);
+    static constexpr size_t smem() {
+        return (size_t)S * XROW + FW_EPI_WARPS * OUT + WBYTES + CO * 4 + (2 * S + 2 * NT) * 8 + 16;
+    }
+};
+
+template <int CI, int CO, int EPI>
+__global__ void __launch_bounds__(FW_THREADS, 1)
+    conv_tc_kernel(const __grid_constant__ CUtensorMap xmap, const uint8_t* __restrict__ x,
+                   const __nv_bfloat16* __restrict__ w, const float* __restrict__ bias, uint8_t* __restrict__ y,
+                   const float* res, const uint8_t* __restrict__ mask, int B, int H, int W, int d,
+                   int* __restrict__ status) {
+    using K = Fw<CI, CO>;
+    constexpr int KB = K::KB, S = K::S, NT = K::NT;
+    constexpr int NC = CI / 8;  // 16-byte chunks per input pixel
+    static_assert(S % FW_HALO_WARPS == 0, "slots owned by one halo warp (a parity wait cannot tell two rounds apart)");
+    static_assert(NT % 2 == 0, "output slots owned by one epilogue group");
+    static_assert(S > 2 * KB && NT > 2 * KB + 1, "rows and outputs open at a time");
+    extern __shared__ __align__(1024) uint8_t smem[];
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+    // [rows][output staging][weights][bias][barriers][tmem slot]
+    const uint32_t sx0 = smem_u32(smem), sstg = sx0 + S * K::XROW, sw0 = sstg + FW_EPI_WARPS * K::OUT;
+    float* s_bias = reinterpret_cast<float*>(smem + S * K::XROW + FW_EPI_WARPS * K::OUT + K::WBYTES);
+    uint64_t* s_bar = reinterpret_cast<uint64_t*>(s_bias + CO);
+    uint32_t* s_tmem = reinterpret_cast<uint32_t*>(s_bar + 2 * S + 2 * NT);
+    const uint32_t bar0 = smem_u32(s_bar);
+    auto full = [&](int s) { return bar0 + 8u * s; };
+    auto empty = [&](int s) { return bar0 + 8u * (S + s); };
+    auto tfull = [&](int s) { return bar0 + 8u * (2 * S + s); };
+    auto tempty = [&](int s) { return bar0 + 8u * (2 * S + NT + s); };
+    if (tid == 0) {
+        for (int s = 0; s < S; ++s) {
+            mbar_init_n(full(s), 1 + 32);  // the TMA issuer's expect_tx and the lanes of a halo warp
+            mbar_init_n(empty(s), 1);
+        }
+        for (int s = 0; s < NT; ++s) {
+            mbar_init_n(tfull(s), 1);
+            mbar_init_n(tempty(s), 128);  // the four warps of an epilogue group
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    }
+    if (warp == FW_MMA_WARP) tmem_alloc(smem_u32(s_tmem), K::TCOLS);
+    fence_before_sync();
+    __syncthreads();
+    fence_after_sync();
+    const uint32_t tmem = __shfl_sync(0xffffffffu, *s_tmem, 0);
+
+    const int rows = H / d, ncb = W / TC_COLS;
+    const long long T = (long long)B * d * ncb * rows;
+    bool ok = true;
+
+    if (warp < FW_EPI_WARPS || warp == FW_MMA_WARP) {
+        // beside the first loads: weights [co][t][ci] -> blocks (dx, 16-channel group) of 3 CO rows
+        // x 32 bytes, swizzled (row bi CO + o of a block holds tap dy = 1 - bi), the bias, and
+        // zeroed output slots
+        constexpr int NTH = 32 * (FW_EPI_WARPS + 1);
+        const int t0 = warp == FW_MMA_WARP ? 32 * FW_EPI_WARPS + lane : tid;
+        for (int i = t0; i < 9 * NC * CO; i += NTH) {
+            const int o = i % CO, rest = i / CO, j = rest % NC, tap = rest / NC;  // tap = 3 bi + dxi
+            const int bi = tap / 3, dxi = tap % 3, t = 3 * (2 - bi) + dxi;
+            const uint4 v = *reinterpret_cast<const uint4*>(w + ((size_t)o * 9 + t) * CI + 8 * j);
+            const uint32_t a = sw0 + (uint32_t)(((dxi * KB + (j >> 1)) * 3 + bi) * CO + o) * 32u + (uint32_t)(j & 1) * 16u;
+            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};\n" ::"r"(swz32(a)), "r"(v.x), "r"(v.y), "r"(v.z),
+                         "r"(v.w)
+                         : "memory");
+        }
+        for (int i = t0; i < CO; i += NTH) s_bias[i] = (EPI != LBM_NN_MASK && bias) ? bias[i] : 0.0f;
+        if (warp < FW_EPI_WARPS) {
+            for (int k = warp >> 2; k < NT; k += 2)
+#pragma unroll
+                for (int c0 = 0; c0 < CO; c0 += 16)
+                    tmem_zero16(tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(k * CO + c0));
+            tmem_wait_st();
+        }
+        fence_proxy_async();  // the weights (generic stores) before the tensor cores read them
+        fence_before_sync();
+        asm volatile("bar.sync 1, %0;\n" ::"n"(NTH) : "memory");
+        fence_after_sync();
+    }
+
+    if (warp == FW_TMA_WARP) {
+        if (lane == 0) {
+            Ring<S> q;
+            Run R = first_run(T, rows);
+            do {
+                const Strip t = strip_of(R.strip, d, ncb);
+                for (int i = 0; i < R.n + 2; ++i, q.next()) {
+                    if (q.round) ok = mbar_wait(empty(q.s), (q.round - 1) & 1);
+                    if (!ok) break;
+                    mbar_arrive_tx(full(q.s), TC_COLS * K::XPB);
+                    tma_load_3d(sx0 + (uint32_t)q.s * K::XROW + HALO * K::XPB, &xmap, 0, t.x0,
+                                strip_row(t, R.r0 - 1 + i, rows, d, H), full(q.s));
+                }
+            } while (ok && next_run(R, rows));
+        }
+        __syncwarp();
+    } else if (warp >= FW_HALO_WARP && warp < FW_HALO_WARP + FW_HALO_WARPS) {
+        // d columns on each side of every row, wrapped, 16 bytes per copy
+        Ring<S> q;
+        Run R = first_run(T, rows);
+        do {
+            const Strip t = strip_of(R.strip, d, ncb);
+            for (int i = 0; i < R.n + 2; ++i, q.next()) {
+                if (q.s % FW_HALO_WARPS != warp - FW_HALO_WARP) continue;
+                if (q.round) ok = mbar_wait(empty(q.s), (q.round - 1) & 1);
+                if (!ok) break;
+                const long long row = strip_row(t, R.r0 - 1 + i, rows, d, H);
+                for (int k = lane; k < 2 * d * NC; k += 32) {
+                    const int jc = k % NC, e = k / NC;
+                    int xx = e < d ? t.x0 - 1 - e : t.x0 + TC_COLS + (e - d);
+                    const int slot = e < d ? HALO - 1 - e : HALO + TC_COLS + (e - d);
+                    xx += xx < 0 ? W : (xx >= W ? -W : 0);
+                    cp_async16(swz<K::XPB>(sx0 + (uint32_t)q.s * K::XROW + (uint32_t)slot * K::XPB + 16u * jc),
+                               x + (row * W + xx) * (16LL * NC) + 16 * jc);
+                }
+                cp_async_commit();
+                cp_async_wait_all();
+                fence_proxy_async();
+                mbar_arrive(full(q.s));
+            }
+        } while (ok && next_run(R, rows));
+    } else if (warp == FW_MMA_WARP) {
+        // The whole warp runs the loop with warp-uniform values (slots, descriptors), one
+        // elected lane issues: with the loop inside a lane's branch the compiler moved
+        // each MMA's five operands into uniform registers one by one.
+        const uint32_t leader = elect_one();
+        const uint32_t xhi = sdesc_hi(K::XPB == 128 ? 1024 : 256, K::XPB == 128 ? LAYOUT_SW128 : LAYOUT_SW32);
+        const uint32_t whi = sdesc_hi(256, LAYOUT_SW32);
+        const uint32_t xl = sdesc_lo(sx0 + (uint32_t)(HALO - d) * K::XPB, 16), wl = sdesc_lo(sw0, 16);
+        // where group kb of the input rows stands: run, row i of its n + 2, ring slot, and
+        // the output slot of its first output row (row i - 2 of the run, or row 0)
+        struct Walk {
+            Run R;
+            Ring<S> q;
+            int i = 0, lo = 0;
+            bool live = true;
+        } at[KB];
+#pragma unroll
+        for (int kb = 0; kb < KB; ++kb) at[kb].R = first_run(T, rows);
+        Ring<NT> fresh;  // the next output slot to open
+        for (int step = 0; ok && at[KB - 1].live; ++step) {
+#pragma unroll
+            for (int kb = 0; kb < KB; ++kb) {
+                Walk& a = at[kb];
+                if (!ok || step < 2 * kb || !a.live) continue;
+                if (kb == 0) {
+                    if (a.i < a.R.n) {
+                        if (fresh.round) ok = mbar_wait(tempty(fresh.s), (fresh.round - 1) & 1);
+                        fresh.next();
+                    }
+                    ok = ok && mbar_wait(full(a.q.s), a.q.round & 1);
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) continue;
+                    fence_after_sync();
+                }
+                // output rows first .. first + c - 1 of the run from slot lo on, the first at
+                // weight block bi (dy = 1 - bi)
+                const int first = a.i < 2 ? 0 : a.i - 2, c = (a.i < a.R.n ? a.i : a.R.n - 1) - first + 1;
+                const int bi = first - (a.i - 2), c1 = a.lo + c > NT ? NT - a.lo : c;
+                const uint32_t row = xl + (uint32_t)a.q.s * (K::XROW / 16) + 2u * kb;
+                auto taps = [&](int slot, int n, int b) {
+                    const uint32_t idesc = idesc_bf16(128, 0, 0, 0) | ((uint32_t)(n * CO >> 3) << 17);
+#pragma unroll
+                    for (int dxi = 0; dxi < 3; ++dxi)
+                        umma_if(leader, tmem + (uint32_t)(slot * CO), row + (uint32_t)(dxi * d) * (K::XPB / 16), xhi,
+                                wl + (uint32_t)(((dxi * KB + kb) * 3 + b) * CO) * 2u, whi, idesc);
+                };
+                taps(a.lo, c1, bi);
+                if (c1 < c) taps(0, c - c1, bi + c1);
+                if (kb == KB - 1) {
+                    commit_if(leader, empty(a.q.s));
+                    if (a.i >= 2) commit_if(leader, tfull(a.lo));
+                }
+                a.q.next();
+                if (a.i >= 2) a.lo = a.lo + 1 == NT ? 0 : a.lo + 1;
+                if (++a.i == a.R.n + 2) {
+                    a.i = 0;
+                    a.live = next_run(a.R, rows);
+                }
+            }
+        }
+        __syncwarp();
+    } else {
+        // ---- epilogue: TMEM lane quarter, pixel x0 + 32 quarter + lane, every other output row
+        const int quarter = warp & 3, group = warp >> 2;
+        const uint32_t stg = sstg + (uint32_t)warp * K::OUT;  // this warp's output staging
+        const uint32_t tq = tmem + ((uint32_t)(32 * quarter) << 16);
+        Ring<NT> o;
+        Run R = first_run(T, rows);
+        do {
+            const Strip t = strip_of(R.strip, d, ncb);
+            for (int j = 0; j < R.n; ++j, o.next()) {
+                if ((o.s & 1) != group) continue;
+                const long long px0 = (long long)strip_row(t, R.r0 + j, rows, d, H) * W + t.x0 + 32 * quarter;
+                // the operands of the epilogue, requested before the wait
+                uint4 mk[EPI == LBM_NN_MASK ? 6 : 1];
+                float4 rs[EPI == LBM_NN_RESIDUAL ? 4 : 1];
+                if constexpr (EPI == LBM_NN_MASK) {
+#pragma unroll
+                    for (int k = 0; k < 6; ++k) mk[k] = __ldg(reinterpret_cast<const uint4*>(mask + (px0 + lane) * 96) + k);
+                }
+                if constexpr (EPI == LBM_NN_RESIDUAL) {
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) rs[k] = reinterpret_cast<const float4*>(res + (px0 + lane) * 16)[k];
+                }
+                ok = mbar_wait(tfull(o.s), o.round & 1);
+                if (!ok) break;
+                fence_after_sync();
+                const uint32_t tb = tq + (uint32_t)(o.s * CO);
+                float v[CO];
+                if constexpr (CO == 48) tmem_ld48(tb, v);
+                else tmem_ld16(tb, v);
+#pragma unroll
+                for (int c0 = 0; c0 < CO; c0 += 16) tmem_zero16(tb + (uint32_t)c0);
+                tmem_wait_st();
+                fence_before_sync();
+                mbar_arrive(tempty(o.s));
+                uint4 out[K::OUT / 512];
+                if constexpr (CO == 48) {
+                    static_assert(EPI == LBM_NN_RELU || EPI == LBM_NN_MASK, "48-channel epilogues: ReLU or mask");
+#pragma unroll
+                    for (int q4 = 0; q4 < 6; ++q4) {
+                        uint32_t u[4];
+                        const uint32_t m[4] = {mk[EPI == LBM_NN_MASK ? q4 : 0].x, mk[EPI == LBM_NN_MASK ? q4 : 0].y,
+                                               mk[EPI == LBM_NN_MASK ? q4 : 0].z, mk[EPI == LBM_NN_MASK ? q4 : 0].w};
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            const int q = 4 * q4 + e;
+                            if constexpr (EPI == LBM_NN_RELU)
+                                u[e] = pack_bf16x2(fmaxf(v[2 * q] + s_bias[2 * q], 0.0f),
+                                                   fmaxf(v[2 * q + 1] + s_bias[2 * q + 1], 0.0f));
+                            else
+                                u[e] = pack_bf16x2(bf16_lo(m[e]) > 0.0f ? v[2 * q] : 0.0f,
+                                                   bf16_hi(m[e]) > 0.0f ? v[2 * q + 1] : 0.0f);
+                        }
+                        out[q4] = make_uint4(u[0], u[1], u[2], u[3]);
+                    }
+                } else {
+                    static_assert(EPI == LBM_NN_RESIDUAL && CO == 16, "16-channel epilogue: residual");
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const float4 a = rs[EPI == LBM_NN_RESIDUAL ? k : 0];
+                        out[k] = make_uint4(__float_as_uint(a.x + v[4 * k] + s_bias[4 * k]),
+                                            __float_as_uint(a.y + v[4 * k + 1] + s_bias[4 * k + 1]),
+                                            __float_as_uint(a.z + v[4 * k + 2] + s_bias[4 * k + 2]),
+                                            __float_as_uint(a.w + v[4 * k + 3] + s_bias[4 * k + 3]));
+                    }
+                }
+                // the warp's 32 pixels are one contiguous run of y: staged, then one bulk store
+                // (after the previous one has read the staging)
+                if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");
+                __syncwarp();
+#pragma unroll
+                for (int k = 0; k < (int)(K::OUT / 512); ++k)
+                    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};\n" ::"r"(stg + (uint32_t)lane * (K::OUT / 32) + 16u * k),
+                                 "r"(out[k].x), "r"(out[k].y), "r"(out[k].z), "r"(out[k].w)
+                                 : "memory");
+                fence_proxy_async();  // the staging (generic stores) before the bulk copy reads it
+                __syncwarp();
+                if (lane == 0) {
+                    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;\n" ::"l"(
+                                     __cvta_generic_to_global(y + px0 * (K::OUT / 32))),
+                                 "r"(stg), "r"(K::OUT)
+                                 : "memory");
+                    asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
+                }
+            }
+        } while (ok && next_run(R, rows));
+        // every store of this warp complete before the CTA (and its staging) goes away
+        if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;\n" ::: "memory");
+    }
+    if (!ok) atomicOr(status, 1);
+    cp_async_wait_all();
+    fence_before_sync();
+    __syncthreads();
+    if (warp == FW_MMA_WARP) {
+        fence_after_sync();
+        tmem_free(tmem, K::TCOLS);
+    }
+}
+
+// Tensor maps of an NHWC bfloat16 activation.
+using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
+                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
+                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+
+EncodeTiledFn encode_tiled() {
+    static EncodeTiledFn fn = nullptr;
+    if (!fn) {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
+                cudaSuccess &&
+            q == cudaDriverEntryPointSuccess)
+            fn = reinterpret_cast<EncodeTiledFn>(p);
+    }
+    return fn;
+}
+
+// {channel, x, image row}, one box per image row of 128 pixels: 48 channels as 128-byte pixel
+// slots (box of 64 channels, the 16 beyond the tensor read as zeros; 128-byte
+// swizzle), 16 channels as 32-byte ones.
+bool row_map(CUtensorMap* map, const void* x, int C, int B, int H, int W) {
+    const EncodeTiledFn fn = encode_tiled();
+    if (!fn) return false;
+    const bool wide = C == 48;
+    const cuuint64_t dims[3] = {(cuuint64_t)C, (cuuint64_t)W, (cuuint64_t)B * H};
+    const cuuint64_t strides[2] = {(cuuint64_t)C * 2, (cuuint64_t)W * C * 2};
+    const cuuint32_t box[3] = {wide ? 64u : 16u, (cuuint32_t)TC_COLS, 1};
+    const cuuint32_t estr[3] = {1, 1, 1};
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(x), dims, strides, box, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, wide ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_32B,
+              CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// ... and one box per image row of 128 pixels as 16-channel planes (32-byte swizzle):
+// {channel of the plane, x, image row, plane}.
+bool plane_map(CUtensorMap* map, const void* x, int C, int B, int H, int W) {
+    const EncodeTiledFn fn = encode_tiled();
+    if (!fn) return false;
+    const cuuint64_t dims[4] = {16, (cuuint64_t)W, (cuuint64_t)B * H, (cuuint64_t)C / 16};
+    const cuuint64_t strides[3] = {(cuuint64_t)C * 2, (cuuint64_t)W * C * 2, 32};
+    const cuuint32_t box[4] = {16, (cuuint32_t)TC_COLS, 1, (cuuint32_t)C / 16};
+    const cuuint32_t estr[4] = {1, 1, 1, 1};
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(x), dims, strides, box, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+template <int CI, int CO, int EPI>
+int conv_tc_launch(const void* x, const void* w, const float* bias, void* y, const float* res, const void* mask, int B,
+                   int H, int W, int d, int* status, cudaStream_t s) {
+    auto k = conv_tc_kernel<CI, CO, EPI>;
+    static_assert(Fw<CI, CO>::smem() <= 227 * 1024, "shared memory");
+    const size_t smem = std::max(Fw<CI, CO>::smem(), TC_MIN_SMEM);
+    CUtensorMap map;
+    if (!row_map(&map, x, CI, B, H, W)) return LBM_ERR_CUDA;
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+        return LBM_ERR_CUDA;
+    const int grid = (int)std::min<long long>((long long)B * H * (W / TC_COLS), (long long)nn_sm_count());
+    k<<<grid, FW_THREADS, smem, s>>>(map, static_cast<const uint8_t*>(x), static_cast<const __nv_bfloat16*>(w), bias,
+                                     static_cast<uint8_t*>(y), res, static_cast<const uint8_t*>(mask), B, H, W, d, status);
+    return cudaGetLastError() == cudaSuccess ? LBM_OK : LBM_ERR_CUDA;
+}
+
+// ------------------------------------------------------ weight gradient --
+// dw[o][t][c] = sum_p dy[p][o] x[p + d off_t][c]: per tap a GEMM with K = pixels,
+// 16 per MMA, both operands read MN-major (channels contiguous) from the rows as the
+// TMA writes them.  A CTA marches down strips of image rows (columns 128 cb .., rows
+// of one residue modulo d): each row of x and of dy is loaded once, and row k of x
+// meets rows k - 1, k, k + 1 of dy while they are in the ring.
+//
+// What bounds it: the tensor cores' operand reads from shared memory and the rate of
+// MMAs, so one MMA carries as many taps as the layouts allow:
+// * N: the three dy rows stacked, 3 CO columns.  dy is stored as 16-channel planes
+//   of 128 pixels (32-byte swizzle), the planes of a row and the rows of the ring
+//   one after another, so that the 16-column groups of N are a constant 4 KB apart.
+// * M: the column taps.  The groups of M step by the dilation, LBO = d pixels: with
+//   48 input channels (64-channel rows of 128 bytes, 128-byte swizzle, the last 16
+//   channels filled with zeros by the TMA) M = 128 covers dx = -1, 0 and M = 64 dx =
+//   +1; with 16 (32-byte rows) M = 64 covers dx = -1, 0, 1 and an unused shift.
+// One box per row of x and dy: the TMA's time goes per box and per pixel row of a
+// box, and 4 KB boxes of 32-byte rows had been the floor (157 ns each).
+// Measured, 48 -> 48 channels, 16 images of 256 x 256: 155 us with one M = 64, N = 48
+// MMA per tap on units of two rows loaded with their halo rows; 52 us so (16 -> 48: 152
+// and 32, 48 -> 16: 151 and 39).
+// The accumulators (3 CO columns per M block) stay in tensor memory for the whole
+// kernel; a CTA writes one partial per tap and a second kernel adds them in a fixed
+// order: deterministic.
+
 template <int CI, int CO>
 struct Wg {
     static constexpr uint32_t XPB = CI == 48 ? 128 : 32;       // bytes of a pixel slot of x
-    static constexpr uint32_t XROW = WG_PITCH * XPB;           // a row of x with its halo slots
+    static constexpr uint32_t XROW = PITCH * XPB;           // a row of x with its halo slots
     static constexpr uint32_t DROW = (CO / 16) * TC_COLS * 32; // a row of dy: planes of 128 pixels
     // slots: the x rings a multiple of the halo warps, so that each owns its slots (a
     // parity wait cannot tell two rounds apart)
@@ -827,7 +775,7 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
                     if (qx.round) ok = mbar_wait(xempty(qx.s), (qx.round - 1) & 1);
                     if (!ok) break;
                     mbar_arrive_tx(xfull(qx.s), TC_COLS * K::XPB);
-                    tma_load_3d(sx0 + (uint32_t)qx.s * K::XROW + WG_HALO * K::XPB, &xmap, 0, t.x0,
+                    tma_load_3d(sx0 + (uint32_t)qx.s * K::XROW + HALO * K::XPB, &xmap, 0, t.x0,
                                 strip_row(t, R.r0 - 1 + i, rows, d, H), xfull(qx.s));
                     qx.next();
                 }
@@ -849,7 +797,7 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
                 for (int k = lane; k < 2 * d * NCX; k += 32) {
                     const int jc = k % NCX, e = k / NCX;
                     int xx = e < d ? t.x0 - 1 - e : t.x0 + TC_COLS + (e - d);
-                    const int slot = e < d ? WG_HALO - 1 - e : WG_HALO + TC_COLS + (e - d);
+                    const int slot = e < d ? HALO - 1 - e : HALO + TC_COLS + (e - d);
                     xx += xx < 0 ? W : (xx >= W ? -W : 0);
                     cp_async16(swz<K::XPB>(sx0 + (uint32_t)qx.s * K::XROW + (uint32_t)slot * K::XPB + 16u * jc),
                                x + (row * W + xx) * (16LL * NCX) + 16 * jc);
@@ -869,7 +817,7 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
         Ring<SD> qd;
         const uint32_t xhi = sdesc_hi(K::XPB == 128 ? 1024 : 256, K::XPB == 128 ? LAYOUT_SW128 : LAYOUT_SW32);
         const uint32_t dhi = sdesc_hi(256, LAYOUT_SW32);
-        const uint32_t xl = sdesc_lo(sx0 + (uint32_t)(WG_HALO - d) * K::XPB, (uint32_t)d * K::XPB);
+        const uint32_t xl = sdesc_lo(sx0 + (uint32_t)(HALO - d) * K::XPB, (uint32_t)d * K::XPB);
         const uint32_t dl = sdesc_lo(sd0, TC_COLS * 32);
         // n3 dy rows from slot s on, at stack position k
         auto stack = [&](int sx, int s, int n3, int k) {
@@ -1021,20 +969,20 @@ int lbm_nn_conv3x3(const void* x, int32_t cin, const void* weights, const float*
     const int d = dilation;
     if (epilogue == LBM_NN_RELU) {
         if (cin == 16 && cout == 48)
-            return conv_tc_dispatch<16, 48, LBM_NN_RELU>(x, weights, bias, y, nullptr, nullptr, batch, h, w, d, status, s);
+            return conv_tc_launch<16, 48, LBM_NN_RELU>(x, weights, bias, y, nullptr, nullptr, batch, h, w, d, status, s);
         if (cin == 48 && cout == 48)
-            return conv_tc_dispatch<48, 48, LBM_NN_RELU>(x, weights, bias, y, nullptr, nullptr, batch, h, w, d, status, s);
+            return conv_tc_launch<48, 48, LBM_NN_RELU>(x, weights, bias, y, nullptr, nullptr, batch, h, w, d, status, s);
     } else if (epilogue == LBM_NN_RESIDUAL) {
         if (!residual) return LBM_ERR_ARG;
         if (cin == 48 && cout == 16)
-            return conv_tc_dispatch<48, 16, LBM_NN_RESIDUAL>(x, weights, bias, y, residual, nullptr, batch, h, w, d,
+            return conv_tc_launch<48, 16, LBM_NN_RESIDUAL>(x, weights, bias, y, residual, nullptr, batch, h, w, d,
                                                              status, s);
     } else if (epilogue == LBM_NN_MASK) {
         if (!mask) return LBM_ERR_ARG;
         if (cin == 48 && cout == 48)
-            return conv_tc_dispatch<48, 48, LBM_NN_MASK>(x, weights, nullptr, y, nullptr, mask, batch, h, w, d, status, s);
+            return conv_tc_launch<48, 48, LBM_NN_MASK>(x, weights, nullptr, y, nullptr, mask, batch, h, w, d, status, s);
         if (cin == 16 && cout == 48)
-            return conv_tc_dispatch<16, 48, LBM_NN_MASK>(x, weights, nullptr, y, nullptr, mask, batch, h, w, d, status, s);
+            return conv_tc_launch<16, 48, LBM_NN_MASK>(x, weights, nullptr, y, nullptr, mask, batch, h, w, d, status, s);
     }
     return LBM_ERR_ARG;
 }
