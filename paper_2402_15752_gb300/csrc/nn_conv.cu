@@ -168,16 +168,17 @@ __device__ __forceinline__ void commit_if(uint32_t go, uint32_t mbar) {
         : "memory");
 }
 
-// Roles of the forward kernel (warp index): 0-7 epilogue (warp w reads TMEM lane
-// quarter w % 4 of the output rows g = w / 4 mod 2), 8 the TMA issuer (lane 0), 9-12
-// halo loaders (warp 9 + h the rows q = h mod 4), 13 the MMA issuer, which also owns
-// the tensor memory.
-constexpr int FW_EPI_WARPS = 8;
-constexpr int FW_TMA_WARP = 8, FW_HALO_WARP = 9, FW_HALO_WARPS = 4, FW_MMA_WARP = 13;
-constexpr int FW_THREADS = 32 * 14;
-// Roles of the weight-gradient kernel: 0-3 epilogue, 4 TMA, 5-7 halo, 8 MMA.
+// Roles of the forward kernel (warp index): 0-11 epilogue (warp w reads TMEM lane
+// quarter w % 4 of every third output row, w / 4), 12 the TMA issuer (lane 0), 13-16
+// halo loaders (warp 13 + h the rows q = h mod 4), 17 the MMA issuer, which also owns
+// the tensor memory.  Three groups of epilogue warps: with two, the mask epilogue's
+// loads showed (58 us against 53).
+constexpr int FW_GROUPS = 3, FW_EPI_WARPS = 4 * FW_GROUPS;
+constexpr int FW_TMA_WARP = FW_EPI_WARPS, FW_HALO_WARP = FW_TMA_WARP + 1, FW_HALO_WARPS = 4;
+constexpr int FW_MMA_WARP = FW_HALO_WARP + FW_HALO_WARPS, FW_THREADS = 32 * (FW_MMA_WARP + 1);
+// Roles of the weight-gradient kernel: 0-3 epilogue, 4 TMA, 5-7 halo, 8-9 MMA.
 constexpr int WG_TMA_WARP = 4, WG_HALO_WARP = 5, WG_HALO_WARPS = 3, WG_MMA_WARP = 8;
-constexpr int WG_THREADS = 32 * 9;
+constexpr int WG_THREADS = 32 * 10;
 // A row in shared memory: HALO halo slots, the 128 pixels of the strip, HALO halo slots
 // (dilation <= HALO); the first pixel sits HALO slots into the row, on a 1024-byte (48
 // channels) or 256-byte (16) boundary, where the swizzle's pattern starts.
@@ -305,12 +306,13 @@ struct Ring {
 // order of a kernel that holds whole units of rows).  So group g of an input row is
 // issued 2 g rows after its first group, when group g - 1 of the next row has been.
 //
-// What bounds it: HBM (a row in and out per output row; the MMAs of a row take about
-// 0.35 us of the 0.55 us that its bytes take).  48 -> 48 channels, 16 images of 256 x
+// What bounds it: the 9 MMAs of a row, which one thread issues about every 85 ns (0.75
+// us a row against the 0.55 us of its bytes; a second issuer would have to share the
+// accumulators, whose order of accumulation is kept).  48 -> 48 channels, 16 images of 256 x
 // 256: units of 4 rows loaded with their 2 halo rows as 18 boxes of 4 KB took 54 us
 // (76 at dilation 8, units of 2 rows) and 66 us (77) with the mask epilogue, bound by
 // the TMA's time per box and pixel row; one box of 128-byte pixel slots per row,
-// loaded once: @F@.
+// loaded once: 46 us at every dilation, 52 with the mask epilogue.
 template <int CI, int CO>
 struct Fw {
     static constexpr int KB = CI / 16;                         // 16-channel groups of the input
@@ -336,7 +338,6 @@ __global__ void __launch_bounds__(FW_THREADS, 1)
     constexpr int KB = K::KB, S = K::S, NT = K::NT;
     constexpr int NC = CI / 8;  // 16-byte chunks per input pixel
     static_assert(S % FW_HALO_WARPS == 0, "slots owned by one halo warp (a parity wait cannot tell two rounds apart)");
-    static_assert(NT % 2 == 0, "output slots owned by one epilogue group");
     static_assert(S > 2 * KB && NT > 2 * KB + 1, "rows and outputs open at a time");
     extern __shared__ __align__(1024) uint8_t smem[];
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
@@ -388,7 +389,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1)
         }
         for (int i = t0; i < CO; i += NTH) s_bias[i] = (EPI != LBM_NN_MASK && bias) ? bias[i] : 0.0f;
         if (warp < FW_EPI_WARPS) {
-            for (int k = warp >> 2; k < NT; k += 2)
+            for (int k = warp >> 2; k < NT; k += FW_GROUPS)
 #pragma unroll
                 for (int c0 = 0; c0 < CO; c0 += 16)
                     tmem_zero16(tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(k * CO + c0));
@@ -443,8 +444,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1)
         } while (ok && next_run(R, rows));
     } else if (warp == FW_MMA_WARP) {
         // The whole warp runs the loop with warp-uniform values (slots, descriptors), one
-        // elected lane issues: with the loop inside a lane's branch the compiler moved
-        // each MMA's five operands into uniform registers one by one.
+        // elected lane issues.
         const uint32_t leader = elect_one();
         const uint32_t xhi = sdesc_hi(K::XPB == 128 ? 1024 : 256, K::XPB == 128 ? LAYOUT_SW128 : LAYOUT_SW32);
         const uint32_t whi = sdesc_hi(256, LAYOUT_SW32);
@@ -503,16 +503,19 @@ __global__ void __launch_bounds__(FW_THREADS, 1)
         }
         __syncwarp();
     } else {
-        // ---- epilogue: TMEM lane quarter, pixel x0 + 32 quarter + lane, every other output row
+        // ---- epilogue: TMEM lane quarter, pixel x0 + 32 quarter + lane, the group's output rows
+        // (a group meets a slot's rounds out of turn, but a row completes after all rows before
+        // it, so a slot is never two rounds behind the one that a group waits for)
         const int quarter = warp & 3, group = warp >> 2;
         const uint32_t stg = sstg + (uint32_t)warp * K::OUT;  // this warp's output staging
         const uint32_t tq = tmem + ((uint32_t)(32 * quarter) << 16);
         Ring<NT> o;
+        int turn = 0;
         Run R = first_run(T, rows);
         do {
             const Strip t = strip_of(R.strip, d, ncb);
-            for (int j = 0; j < R.n; ++j, o.next()) {
-                if ((o.s & 1) != group) continue;
+            for (int j = 0; j < R.n; ++j, o.next(), turn = turn + 1 == FW_GROUPS ? 0 : turn + 1) {
+                if (turn != group) continue;
                 const long long px0 = (long long)strip_row(t, R.r0 + j, rows, d, H) * W + t.x0 + 32 * quarter;
                 // the operands of the epilogue, requested before the wait
                 uint4 mk[EPI == LBM_NN_MASK ? 6 : 1];
@@ -545,12 +548,18 @@ __global__ void __launch_bounds__(FW_THREADS, 1)
                         uint32_t u[4];
                         const uint32_t m[4] = {mk[EPI == LBM_NN_MASK ? q4 : 0].x, mk[EPI == LBM_NN_MASK ? q4 : 0].y,
                                                mk[EPI == LBM_NN_MASK ? q4 : 0].z, mk[EPI == LBM_NN_MASK ? q4 : 0].w};
+                        float bq[8] = {};
+                        if constexpr (EPI == LBM_NN_RELU) {
+                            const float4 b0 = *reinterpret_cast<const float4*>(s_bias + 8 * q4);
+                            const float4 b1 = *reinterpret_cast<const float4*>(s_bias + 8 * q4 + 4);
+                            bq[0] = b0.x; bq[1] = b0.y; bq[2] = b0.z; bq[3] = b0.w;
+                            bq[4] = b1.x; bq[5] = b1.y; bq[6] = b1.z; bq[7] = b1.w;
+                        }
 #pragma unroll
                         for (int e = 0; e < 4; ++e) {
                             const int q = 4 * q4 + e;
                             if constexpr (EPI == LBM_NN_RELU)
-                                u[e] = pack_bf16x2(fmaxf(v[2 * q] + s_bias[2 * q], 0.0f),
-                                                   fmaxf(v[2 * q + 1] + s_bias[2 * q + 1], 0.0f));
+                                u[e] = pack_bf16x2(fmaxf(v[2 * q] + bq[2 * e], 0.0f), fmaxf(v[2 * q + 1] + bq[2 * e + 1], 0.0f));
                             else
                                 u[e] = pack_bf16x2(bf16_lo(m[e]) > 0.0f ? v[2 * q] : 0.0f,
                                                    bf16_hi(m[e]) > 0.0f ? v[2 * q + 1] : 0.0f);
@@ -684,8 +693,8 @@ int conv_tc_launch(const void* x, const void* w, const float* bias, void* y, con
 // One box per row of x and dy: the TMA's time goes per box and per pixel row of a
 // box, and 4 KB boxes of 32-byte rows had been the floor (157 ns each).
 // Measured, 48 -> 48 channels, 16 images of 256 x 256: 155 us with one M = 64, N = 48
-// MMA per tap on units of two rows loaded with their halo rows; 52 us so (16 -> 48: 152
-// and 32, 48 -> 16: 151 and 39).
+// MMA per tap on units of two rows loaded with their halo rows; 48 us so (16 -> 48: 152
+// and 33, 48 -> 16: 151 and 38).
 // The accumulators (3 CO columns per M block) stay in tensor memory for the whole
 // kernel; a CTA writes one partial per tap and a second kernel adds them in a fixed
 // order: deterministic.
@@ -698,6 +707,9 @@ struct Wg {
     // slots: the x rings a multiple of the halo warps, so that each owns its slots (a
     // parity wait cannot tell two rounds apart)
     static constexpr int SX = CI == 48 ? 6 : 9, SD = 9;
+    // MMA issuers: one per M block, on accumulators of its own (a thread issues an MMA
+    // only about every 100 cycles; two warps overlap: 52 -> 48 us)
+    static constexpr int NI = CI == 48 ? 2 : 1;
     static constexpr uint32_t N3 = 3 * CO;
     static constexpr uint32_t TCOLS = pow2_cols(CI == 48 ? 2 * N3 : N3);
     static constexpr size_t smem() { return (size_t)SX * XROW + SD * DROW + (2 * SX + 2 * SD + 1) * 8 + 16; }
@@ -727,13 +739,13 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
     if (tid == 0) {
         for (int s = 0; s < SX; ++s) {
             mbar_init_n(xfull(s), 1 + 32);  // the TMA issuer's expect_tx and the lanes of a halo warp
-            mbar_init_n(xempty(s), 1);
+            mbar_init_n(xempty(s), K::NI);
         }
         for (int s = 0; s < SD; ++s) {
             mbar_init_n(dfull(s), 1);
-            mbar_init_n(dempty(s), 1);
+            mbar_init_n(dempty(s), K::NI);
         }
-        mbar_init_n(done, 1);
+        mbar_init_n(done, K::NI);
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
     if (warp == WG_MMA_WARP) tmem_alloc(smem_u32(s_tmem), K::TCOLS);
@@ -808,28 +820,26 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
                 mbar_arrive(xfull(qx.s));
             }
         } while (ok && next_run(R, rows));
-    } else if (warp == WG_MMA_WARP) {
-        // The whole warp runs the loop with warp-uniform values (slots, descriptors), one
-        // elected lane issues: with the loop inside a lane's branch the compiler moved
-        // each MMA's five operands into uniform registers one by one.
+    } else if (warp >= WG_MMA_WARP && warp < WG_MMA_WARP + K::NI) {
+        // CI = 48: the first issuer dx = -1, 0 (M = 128), the second dx = +1 (M = 64);
+        // CI = 16: one issuer, all dx (M = 64).  The whole warp runs the loop with
+        // warp-uniform values (slots, descriptors), one elected lane issues.
+        const int part = warp - WG_MMA_WARP;
         const uint32_t leader = elect_one();
         Ring<SX> qx;
         Ring<SD> qd;
         const uint32_t xhi = sdesc_hi(K::XPB == 128 ? 1024 : 256, K::XPB == 128 ? LAYOUT_SW128 : LAYOUT_SW32);
         const uint32_t dhi = sdesc_hi(256, LAYOUT_SW32);
-        const uint32_t xl = sdesc_lo(sx0 + (uint32_t)(HALO - d) * K::XPB, (uint32_t)d * K::XPB);
-        const uint32_t dl = sdesc_lo(sd0, TC_COLS * 32);
+        const uint32_t xl = sdesc_lo(sx0 + (uint32_t)(HALO + (part == 0 ? -d : d)) * K::XPB, (uint32_t)d * K::XPB);
+        const uint32_t dl = sdesc_lo(sd0, TC_COLS * 32), block = tmem + (uint32_t)part * K::N3;
+        const uint32_t shape = idesc_bf16(CI == 48 && part == 0 ? 128 : 64, 0, 1, 1);
         // n3 dy rows from slot s on, at stack position k
         auto stack = [&](int sx, int s, int n3, int k) {
-            const uint32_t i1 = idesc_bf16(CI == 48 ? 128 : 64, 0, 1, 1) | ((uint32_t)(n3 * CO >> 3) << 17);
-            const uint32_t i2 = idesc_bf16(64, 0, 1, 1) | ((uint32_t)(n3 * CO >> 3) << 17);
+            const uint32_t idesc = shape | ((uint32_t)(n3 * CO >> 3) << 17);
             uint32_t a = xl + (uint32_t)sx * (K::XROW / 16), b = dl + (uint32_t)s * (K::DROW / 16);
-            const uint32_t a2 = (uint32_t)(2 * d) * (K::XPB / 16);
-            const uint32_t c = tmem + (uint32_t)(k * CO);
 #pragma unroll
             for (int p0 = 0; p0 < TC_COLS; p0 += 16) {
-                umma_if(leader, c, a, xhi, b, dhi, i1);
-                if constexpr (CI == 48) umma_if(leader, c + K::N3, a + a2, xhi, b, dhi, i2);
+                umma_if(leader, block + (uint32_t)(k * CO), a, xhi, b, dhi, idesc);
                 a += K::XPB;  // 16 pixels, in 16-byte units
                 b += 32;
             }
@@ -861,7 +871,7 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
         } while (ok && next_run(R, rows));
         commit_if(leader, done);
         __syncwarp();
-    } else {
+    } else if (warp < 4) {
         // ---- epilogue: stack position k of the columns is tap row dy = 1 - k
         ok = mbar_wait(done, 0);
         fence_after_sync();

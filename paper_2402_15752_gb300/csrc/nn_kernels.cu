@@ -118,6 +118,19 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
     e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
 }
 
+// A pixel's squares and gradient formed in double throughout (a call, so that the
+// common path holds none of it: predicated off, it kept the FP64 pipe busy).
+__device__ __noinline__ double pixel_in_double(const float* __restrict__ x, const float* __restrict__ y, int U,
+                                               double two_inv, __nv_bfloat16* __restrict__ out) {
+    double a = 0.0;
+    for (int c = 0; c < 16; ++c) {
+        const double d = c < U ? (double)x[c] - (double)y[c] : 0.0;
+        a += d * d;
+        if (out) out[c] = __float2bfloat16_rn((float)(two_inv * d));
+    }
+    return a;
+}
+
 // VEC: pred, target and dpred on 16-byte boundaries (else scalar accesses).
 // dpred = 2 inv d: the FP32 product with 2 inv = khi + klo, accurate to 2^-46 before
 // its one rounding to float, then rounded to bfloat16.
@@ -147,30 +160,28 @@ __global__ void __launch_bounds__(256)
     auto pixel = [&](long long p, const float (&x)[4 * NV], const float (&y)[4 * NV]) {
         float g[16] = {};
         float H = 0.0f, L = 0.0f;
-        double far = 0.0;  // squares outside the float range
+        bool odd = false;  // a difference whose square leaves the float range
 #pragma unroll
         for (int c = 0; c < 4 * NV; ++c) {
             if (c >= U) continue;
             float s, e;
             two_sum(x[c], -y[c], s, e);
             const float m = fabsf(s);
-            if (m == 0.0f || (m > 1e-14f && m < 1e18f)) {
-                const float h = __fmul_rn(s, s);
-                // the product's error, and the cross term of the split
-                const float l = __fadd_rn(__fmaf_rn(s, s, -h), __fmul_rn(2.0f * s, e));
-                float z, r;
-                two_sum(H, h, z, r);
-                H = z;
-                L = __fadd_rn(L, __fadd_rn(r, l));
-                g[c] = __fmaf_rn(khi, s, __fmaf_rn(khi, e, __fmul_rn(klo, s)));
-            } else {
-                const double d = (double)x[c] - (double)y[c];
-                far += d * d;
-                g[c] = (float)(2.0 * inv * d);
-            }
+            odd |= !(m == 0.0f || (m > 1e-14f && m < 1e18f));  // also NaN
+            const float h = __fmul_rn(s, s);
+            // the product's error, and the cross term of the split
+            const float l = __fadd_rn(__fmaf_rn(s, s, -h), __fmul_rn(2.0f * s, e));
+            float z, r;
+            two_sum(H, h, z, r);
+            H = z;
+            L = __fadd_rn(L, __fadd_rn(r, l));
+            g[c] = __fmaf_rn(khi, s, __fmaf_rn(khi, e, __fmul_rn(klo, s)));
         }
-        a += ((double)H + (double)L);
-        if (far != 0.0) a += far;  // also NaN
+        if (odd) {
+            a += pixel_in_double(pred + p * 16, target + p * 16, U, 2.0 * inv, dpred ? dpred + p * 16 : nullptr);
+            return;
+        }
+        a += (double)H + (double)L;
         if (!dpred) return;
         if constexpr (VEC) {
             uint32_t out[8];
