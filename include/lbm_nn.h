@@ -61,6 +61,15 @@ int lbm_nn_conv3x3_wgrad(const void* x, int32_t cin, const void* dy, int32_t cou
                          void* partials, size_t partial_bytes, int32_t batch, int32_t h,
                          int32_t w, int32_t dilation, int32_t* status, void* stream);
 
+/* The same, and the bias gradient db[o] = sum over pixels of dy[., o] from the rows of
+ * dy that the weight gradient holds (no second pass over dy).  bias_partials: cout
+ * floats per partial of dw (as partial_bytes: at most SMs * cout floats); db may be
+ * NULL (weights only). */
+int lbm_nn_conv3x3_wgrad_bias(const void* x, int32_t cin, const void* dy, int32_t cout, float* dw,
+                              float* db, void* partials, size_t partial_bytes,
+                              float* bias_partials, int32_t batch, int32_t h, int32_t w,
+                              int32_t dilation, int32_t* status, void* stream);
+
 /* Bias gradient db[o] = sum over pixels of dy[., o] (float, overwritten), fixed
  * order through `partials` (>= 1024 * cout floats). */
 int lbm_nn_bias_grad(const void* dy, int32_t cout, int64_t pixels, float* db, float* partials,

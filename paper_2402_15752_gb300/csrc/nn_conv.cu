@@ -718,8 +718,8 @@ struct Wg {
 template <int CI, int CO>
 __global__ void __launch_bounds__(WG_THREADS, 1)
     wgrad_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap dmap,
-                    const uint8_t* __restrict__ x, float* __restrict__ partials, int B, int H, int W, int d,
-                    int* __restrict__ status) {
+                    const uint8_t* __restrict__ x, float* __restrict__ partials, float* __restrict__ bpart, int B, int H,
+                    int W, int d, int* __restrict__ status) {
     using K = Wg<CI, CO>;
     constexpr int SX = K::SX, SD = K::SD;
     constexpr int NCX = CI / 8;  // 16-byte chunks of an x pixel
@@ -743,7 +743,7 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
         }
         for (int s = 0; s < SD; ++s) {
             mbar_init_n(dfull(s), 1);
-            mbar_init_n(dempty(s), K::NI);
+            mbar_init_n(dempty(s), K::NI + (bpart ? 4 : 0));  // the issuers, and the warps that sum the bias gradient
         }
         mbar_init_n(done, K::NI);
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
@@ -872,9 +872,54 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
         commit_if(leader, done);
         __syncwarp();
     } else if (warp < 4) {
+        // ---- the bias gradient, while the issuers run: thread tid sums the channels of its pixel
+        // of every dy row from the ring
+        float a[CO] = {};
+        if (bpart) {
+            Ring<SD> qd;
+            Run R = first_run(T, rows);
+            do {
+                for (int i = 0; i < R.n; ++i, qd.next()) {
+                    ok = mbar_wait(dfull(qd.s), qd.round & 1);
+                    if (!ok) break;
+                    const uint32_t px = sd0 + (uint32_t)qd.s * K::DROW + 32u * tid;
+#pragma unroll
+                    for (int c = 0; c < CO / 8; ++c) {
+                        uint32_t v[4];
+                        asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];\n"
+                                     : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
+                                     : "r"(swz32(px + (uint32_t)(c >> 1) * (TC_COLS * 32) + 16u * (c & 1)))
+                                     : "memory");
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            a[8 * c + 2 * e] += bf16_lo(v[e]);
+                            a[8 * c + 2 * e + 1] += bf16_hi(v[e]);
+                        }
+                    }
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(dempty(qd.s));
+                }
+            } while (ok && next_run(R, rows));
+#pragma unroll
+            for (int c = 0; c < CO; ++c) {
+#pragma unroll
+                for (int off = 16; off > 0; off >>= 1) a[c] += __shfl_down_sync(0xffffffffu, a[c], off);
+            }
+        }
         // ---- epilogue: stack position k of the columns is tap row dy = 1 - k
-        ok = mbar_wait(done, 0);
+        ok = mbar_wait(done, 0) && ok;
         fence_after_sync();
+        if (bpart) {
+            // the warps' sums meet where the rows were (all of them have been used)
+            float* s_sum = reinterpret_cast<float*>(smem);
+            if (lane == 0)
+#pragma unroll
+                for (int c = 0; c < CO; ++c) s_sum[warp * CO + c] = a[c];
+            asm volatile("bar.sync 1, 128;\n" ::: "memory");
+            if (tid < CO)
+                bpart[(size_t)blockIdx.x * CO + tid] =
+                    (s_sum[tid] + s_sum[CO + tid]) + (s_sum[2 * CO + tid] + s_sum[3 * CO + tid]);
+        }
         float* out = partials + (size_t)blockIdx.x * 9 * CI * CO;
         const uint32_t tq = tmem + ((uint32_t)(32 * warp) << 16);
         auto write = [&](uint32_t block, int dxi, int ci, bool mine) {
@@ -914,18 +959,23 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
 // takes 32 consecutive outputs (128 contiguous bytes of a partial) and deals the
 // partials to 8 warps, whose sums it adds in order (44 us for 152 partials of 9 x 48
 // x 48 when one thread added all of an output's partials; 6.2 us so).
+// The blocks beyond those of dw add the bias gradient's partials alike.
 constexpr int WR_OUT = 32, WR_SEG = 8;
 __global__ void __launch_bounds__(WR_OUT * WR_SEG)
-    wgrad_tc_reduce(const float* __restrict__ partials, int nb, int CO, int CI, float* __restrict__ dw) {
-    const int n = 9 * CO * CI;
+    wgrad_tc_reduce(const float* __restrict__ partials, int nb, int CO, int CI, float* __restrict__ dw,
+                    const float* __restrict__ bpart, float* __restrict__ db) {
+    const int wblocks = (9 * CO * CI + WR_OUT - 1) / WR_OUT;
+    const bool bias = (int)blockIdx.x >= wblocks;
+    const int n = bias ? CO : 9 * CO * CI;
+    const float* __restrict__ src = bias ? bpart : partials;
     __shared__ float s[WR_SEG][WR_OUT];
     const int k = threadIdx.x % WR_OUT, seg = threadIdx.x / WR_OUT;
-    const int i = blockIdx.x * WR_OUT + k;
+    const int i = ((int)blockIdx.x - (bias ? wblocks : 0)) * WR_OUT + k;
     float a = 0.0f;
     if (i < n) {
         const int per = (nb + WR_SEG - 1) / WR_SEG, b1 = min(nb, (seg + 1) * per);
 #pragma unroll 8
-        for (int b = seg * per; b < b1; ++b) a += __ldg(partials + (size_t)b * n + i);
+        for (int b = seg * per; b < b1; ++b) a += __ldg(src + (size_t)b * n + i);
     }
     s[seg][k] = a;
     __syncthreads();
@@ -934,7 +984,8 @@ __global__ void __launch_bounds__(WR_OUT * WR_SEG)
 #pragma unroll
         for (int j = 0; j < WR_SEG; ++j) t += s[j][k];
         const int c = i % CI, o = (i / CI) % CO, tap = i / (CI * CO);
-        dw[((size_t)o * 9 + tap) * CI + c] = t;
+        if (bias) db[i] = t;
+        else dw[((size_t)o * 9 + tap) * CI + c] = t;
     }
 }
 
@@ -945,8 +996,8 @@ long long wgrad_parts(int B, int H, int W, int d) {
 }
 
 template <int CI, int CO>
-int wgrad_tc_launch(const void* x, const void* dy, float* dw, float* part, int B, int H, int W, int d, int* status,
-                    cudaStream_t s) {
+int wgrad_tc_launch(const void* x, const void* dy, float* dw, float* db, float* part, float* bpart, int B, int H, int W,
+                    int d, int* status, cudaStream_t s) {
     auto k = wgrad_tc_kernel<CI, CO>;
     static_assert(Wg<CI, CO>::smem() <= 227 * 1024, "shared memory");
     const size_t smem = std::max(Wg<CI, CO>::smem(), TC_MIN_SMEM);
@@ -955,8 +1006,9 @@ int wgrad_tc_launch(const void* x, const void* dy, float* dw, float* part, int B
     if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return LBM_ERR_CUDA;
     const int grid = (int)std::min<long long>(wgrad_parts(B, H, W, d), (long long)nn_sm_count());
-    k<<<grid, WG_THREADS, smem, s>>>(xmap, dmap, static_cast<const uint8_t*>(x), part, B, H, W, d, status);
-    wgrad_tc_reduce<<<(9 * CO * CI + WR_OUT - 1) / WR_OUT, WR_OUT * WR_SEG, 0, s>>>(part, grid, CO, CI, dw);
+    k<<<grid, WG_THREADS, smem, s>>>(xmap, dmap, static_cast<const uint8_t*>(x), part, db ? bpart : nullptr, B, H, W, d, status);
+    const int blocks = (9 * CO * CI + WR_OUT - 1) / WR_OUT + (db ? (CO + WR_OUT - 1) / WR_OUT : 0);
+    wgrad_tc_reduce<<<blocks, WR_OUT * WR_SEG, 0, s>>>(part, grid, CO, CI, dw, bpart, db);
     return cudaGetLastError() == cudaSuccess ? LBM_OK : LBM_ERR_CUDA;
 }
 
@@ -1002,19 +1054,30 @@ size_t lbm_nn_wgrad_partial_bytes(int32_t cin, int32_t cout, int32_t batch, int3
     return (size_t)std::min<long long>(wgrad_parts(batch, h, w, dilation), (long long)nn_sm_count()) * 9 * cin * cout * sizeof(float);
 }
 
-int lbm_nn_conv3x3_wgrad(const void* x, int32_t cin, const void* dy, int32_t cout, float* dw, void* partials,
-                         size_t partial_bytes, int32_t batch, int32_t h, int32_t w, int32_t dilation, int32_t* status,
-                         void* stream) {
+int lbm_nn_conv3x3_wgrad_bias(const void* x, int32_t cin, const void* dy, int32_t cout, float* dw, float* db,
+                              void* partials, size_t partial_bytes, float* bias_partials, int32_t batch, int32_t h,
+                              int32_t w, int32_t dilation, int32_t* status, void* stream) {
     if (!x || !dy || !dw || !partials || !status || !conv_shape_ok(batch, h, w, dilation)) return LBM_ERR_ARG;
+    if (db && !bias_partials) return LBM_ERR_ARG;
     if (((uintptr_t)x | (uintptr_t)dy) % 16 != 0) return LBM_ERR_ARG;
     if (partial_bytes < lbm_nn_wgrad_partial_bytes(cin, cout, batch, h, w, dilation)) return LBM_ERR_ARG;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     float* part = static_cast<float*>(partials);
     const int d = dilation;
-    if (cin == 16 && cout == 48) return wgrad_tc_launch<16, 48>(x, dy, dw, part, batch, h, w, d, status, s);
-    if (cin == 48 && cout == 48) return wgrad_tc_launch<48, 48>(x, dy, dw, part, batch, h, w, d, status, s);
-    if (cin == 48 && cout == 16) return wgrad_tc_launch<48, 16>(x, dy, dw, part, batch, h, w, d, status, s);
+    if (cin == 16 && cout == 48)
+        return wgrad_tc_launch<16, 48>(x, dy, dw, db, part, bias_partials, batch, h, w, d, status, s);
+    if (cin == 48 && cout == 48)
+        return wgrad_tc_launch<48, 48>(x, dy, dw, db, part, bias_partials, batch, h, w, d, status, s);
+    if (cin == 48 && cout == 16)
+        return wgrad_tc_launch<48, 16>(x, dy, dw, db, part, bias_partials, batch, h, w, d, status, s);
     return LBM_ERR_ARG;
+}
+
+int lbm_nn_conv3x3_wgrad(const void* x, int32_t cin, const void* dy, int32_t cout, float* dw, void* partials,
+                         size_t partial_bytes, int32_t batch, int32_t h, int32_t w, int32_t dilation, int32_t* status,
+                         void* stream) {
+    return lbm_nn_conv3x3_wgrad_bias(x, cin, dy, cout, dw, nullptr, partials, partial_bytes, nullptr, batch, h, w,
+                                     dilation, status, stream);
 }
 
 }  // extern "C"

@@ -55,6 +55,7 @@ def nn_lib():
         "lbm_nn_conv3x3": [vp, i32, vp, vp, i32, i32, vp, vp, vp, i32, i32, i32, i32, vp, vp],
         "lbm_nn_flip_weights": [vp, i32, i32, vp, vp],
         "lbm_nn_conv3x3_wgrad": [vp, i32, vp, i32, vp, vp, sz, i32, i32, i32, i32, vp, vp],
+        "lbm_nn_conv3x3_wgrad_bias": [vp, i32, vp, i32, vp, vp, vp, sz, vp, i32, i32, i32, i32, vp, vp],
         "lbm_nn_bias_grad": [vp, i32, i64, vp, vp, vp],
         "lbm_nn_mse": [vp, vp, i32, i64, vp, vp, vp, vp],
         "lbm_nn_adam": [vp, vp, vp, vp, vp, vp, i64, f32, f32, f32, f32, i32, vp],
@@ -197,7 +198,6 @@ class Net:
         network's input: the residual path dz16 plus layer 0's adjoint
         convolution of its output gradient (the residual epilogue adds them)."""
         L = nn_lib()
-        P = B * H * W
         wpart, bpart = scratch
         dz = dz16
         if dx32 is not None:
@@ -206,9 +206,8 @@ class Net:
             ci, co = LAYERS[l]
             a_l = x16 if l == 0 else acts[l - 1]
             nb = L.lbm_nn_wgrad_partial_bytes(ci, co, B, H, W, self.dil[l])
-            _ck(L.lbm_nn_conv3x3_wgrad(_p(a_l), ci, _p(dz), co, _p(self.gw[l]), _p(wpart), nb, B, H, W,
-                                       self.dil[l], _p(self.status), self.s), "wgrad%d" % l)
-            _ck(L.lbm_nn_bias_grad(_p(dz), co, P, _p(self.gb[l]), _p(bpart), self.s), "bgrad%d" % l)
+            _ck(L.lbm_nn_conv3x3_wgrad_bias(_p(a_l), ci, _p(dz), co, _p(self.gw[l]), _p(self.gb[l]), _p(wpart), nb,
+                                            _p(bpart), B, H, W, self.dil[l], _p(self.status), self.s), "wgrad%d" % l)
             if l > 0:
                 nxt = dbuf[l % 2]
                 _ck(L.lbm_nn_conv3x3(_p(dz), co, _p(self.wt[l]), None, ci, MASK, None, _p(a_l), _p(nxt),

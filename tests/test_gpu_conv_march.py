@@ -69,4 +69,11 @@ def test_convolution_and_weight_gradient(ci, co, B, H, W, d):
     want = _wgrad(torch, x.double(), dy.double(), d)
     size = _wgrad(torch, x.double().abs(), dy.double().abs(), d)
     assert bool(((dw.double() - want).abs() <= ACC * size).all())
+    # with the bias gradient: the same weight gradient, bit for bit
+    dw2, db = torch.full_like(dw, float("nan")), torch.full((co,), float("nan"), device="cuda")
+    bpart = torch.full((nb // (36 * ci),), float("nan"), device="cuda")
+    assert L.lbm_nn_conv3x3_wgrad_bias(_p(x), ci, _p(dy), co, _p(dw2), _p(db), _p(part), nb, _p(bpart), B, H, W, d,
+                                       _p(st), s) == 0
+    assert torch.equal(dw, dw2)
+    assert bool(((db.double() - dy.double().sum((0, 1, 2))).abs() <= ACC * dy.double().abs().sum((0, 1, 2))).all())
     assert int(st.item()) == 0
