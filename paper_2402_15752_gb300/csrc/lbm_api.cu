@@ -164,6 +164,37 @@ static int choose_strip_height(const lbm_handle* h) {
     return best_h;
 }
 
+// Whether the step runs tiles (tile_kernel, tile64_kernel) instead of strips.  Times
+// are microseconds per step, strips against tiles, on square periodic lattices:
+// * FP64 always: 64^2 82 : 14, 512^2 275 : 165, 1024^2 938 : 622 (D2Q5).  Tiles of 8 x 4
+//   nodes while they leave SMs idle or nearly so (64^2: 13.9 against 15.2 with 16 x 8),
+//   else 16 x 8, whose ring is smaller (128^2: 15.3 against 16.2, 512^2: 165 : 174).
+// * D2Q9 scalars always: the strip kernel spills and holds 34 KB of shared memory per
+//   CTA (FP32 64^2 16.4 : 3.4, 1448^2 191 : 121, 2896^2 704 : 466; bfloat16 64^2 24 : 4.1,
+//   2896^2 563 : 533).
+// * D2Q5 while the strips' serial rows show: FP32 64^2 11.6 : 3.4, 512^2 18.0 : 11.8, 724^2
+//   29.7 : 28.3, then 1024^2 50.7 : 52.3, 2048^2 179 : 194; bfloat16 64^2 20 : 4.0, 512^2
+//   27 : 18, 1024^2 65 : 64, then 1448^2 125 : 126, 2048^2 239 : 246.  Beyond that where
+//   the strips' last 128 columns idle more than the tiles cost (8 %, 16-bit storage 4 %).
+// Tiles address within a row of blocks by 32-bit offsets, and by grid.y.
+static int choose_tiles(const lbm_handle* h) {
+    const lbm_params& p = h->p;
+    const long long nx = p.nx, ny = p.ny, nodes = nx * ny;
+    const bool half = h->L.elem == 2;
+    const long long words = (long long)(half ? h->L.pop_elems / 2 : h->L.pop_elems);
+    if (words >= (1LL << 31) || (ny + 3) / 4 > 65535) return 0;
+    if (p.precision == LBM_FP64) {
+        int sms = 0;
+        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device) != cudaSuccess || sms <= 0) sms = 1;
+        return ((nx + 7) / 8) * ((ny + 3) / 4) <= 2LL * sms ? 1 : 2;
+    }
+    if (p.scalar_q == 9) return 1;
+    if (nodes <= (half ? 1500000 : 700000)) return 1;
+    const long long strips = (nx + lbm::STRIP_W - 1) / lbm::STRIP_W * lbm::STRIP_W * ny;
+    const long long tiles = (nx + 31) / 32 * 32 * ((ny + 3) / 4 * 4);
+    return 100 * strips > (half ? 104 : 108) * tiles;
+}
+
 // Debug build: the readers of the status words of every translation unit with
 // checked kernels (registered during static initialisation).
 namespace lbm {
@@ -238,6 +269,7 @@ int lbm_create(const lbm_params* params, void* d_workspace, size_t workspace_byt
     }
     *h->h_status = 0u;
     h->geo.strip_h = choose_strip_height(h);
+    h->geo.tiled = choose_tiles(h);
     *out = h;
     return LBM_OK;
 }

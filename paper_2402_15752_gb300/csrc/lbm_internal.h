@@ -62,6 +62,7 @@ struct Geometry {
     int nx, ny, nxb;
     int wall_x, wall_y;
     int strip_h;     // rows per CTA of the step kernel
+    int tiled;       // the step runs one tile of nodes per CTA instead of strips (FP64: 1 small, 2 large tiles)
     int one_scalar;  // one-scalar model: h1 planes hold h3, h2 planes unused
     int grad_scheme; // 0: stencils (Eq. 41); 1: local grad c (Eq. 39); 2: also local grad phi
     // 16-bit storage only (else NULL): the bases of the node that wrote each
