@@ -102,6 +102,11 @@ struct lbm_batch {
     bool failed = false;        // a wait gave up: the lattices are out of step
     cudaGraphExec_t graph = nullptr;
     bool graph_tried = false;
+    // one launch per step over tiles of TILE_W x TILE_H (table in d_tiles) instead of the
+    // persistent kernel; its 32-step graphs by the parity of the first step
+    bool per_step = false;
+    int fine_tiles = 0;
+    cudaGraphExec_t step_graph[2] = {};
     // pinned staging of the case descriptors; the event marks the end of the
     // last copy out of it, so a reset rewrites it only once that copy is done
     lbm::BatchCase* h_cases = nullptr;
@@ -169,6 +174,10 @@ struct lbm_batch {
         if (graph) cudaGraphExecDestroy(graph);
         graph = nullptr;
         graph_tried = false;
+        for (auto& g : step_graph) {
+            if (g) cudaGraphExecDestroy(g);
+            g = nullptr;
+        }
     }
 
     lbm::BatchArgs args(int nsteps) const {
@@ -229,6 +238,39 @@ struct lbm_batch {
     }
 
     cudaError_t launch_steps(int n) { return launch(args(n), stream); }
+
+    cudaError_t launch_fine(int64_t t, cudaStream_t s) {
+        return q == 5 ? lbm::launch_batch_tiles<5>(d_cases(), d_tiles(), fine_tiles, t, s)
+                      : lbm::launch_batch_tiles<9>(d_cases(), d_tiles(), fine_tiles, t, s);
+    }
+
+    // nsteps steps as launches, full runs of GRAPH_STEPS from a captured graph
+    cudaError_t step_fine(int64_t nsteps) {
+        constexpr int G = lbm::detail::GRAPH_STEPS;
+        cudaError_t e = cudaSuccess;
+        int64_t done = 0;
+        for (; e == cudaSuccess && nsteps - done >= G; done += G) {
+            cudaGraphExec_t& exec = step_graph[(steps + done) & 1];
+            if (!exec) {
+                cudaStream_t cap = nullptr;
+                cudaGraph_t g = nullptr;
+                e = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking);
+                if (e == cudaSuccess) e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
+                if (e == cudaSuccess) {
+                    cudaError_t le = cudaSuccess;
+                    for (int k = 0; k < G && le == cudaSuccess; ++k) le = launch_fine(steps + done + k, cap);
+                    e = cudaStreamEndCapture(cap, &g);
+                    if (le != cudaSuccess) e = le;
+                }
+                if (e == cudaSuccess) e = cudaGraphInstantiate(&exec, g, 0);
+                if (g) cudaGraphDestroy(g);
+                if (cap) cudaStreamDestroy(cap);
+            }
+            if (e == cudaSuccess) e = cudaGraphLaunch(exec, stream);
+        }
+        for (; e == cudaSuccess && done < nsteps; ++done) e = launch_fine(steps + done, stream);
+        return e;
+    }
 
     // A graph of one GRAPH_STEPS-step launch; falls back to plain launches if the
     // cooperative launch cannot be captured.
@@ -338,6 +380,7 @@ int build_tiling(lbm_batch* b, int tile_w, int tile_h) {
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);  // the vectors are pageable
     if (e != cudaSuccess) return b->fail(LBM_ERR_CUDA, "lbm_batch_set_tiling", e);
     b->drop_graph();
+    b->per_step = false;
     b->tile_w = tile_w;
     b->tile_h = tile_h;
     b->ntiles = (int)tiles.size();
@@ -345,6 +388,38 @@ int build_tiling(lbm_batch* b, int tile_w, int tile_h) {
     b->launch = launch;
     e = b->reset_counters();
     if (e != cudaSuccess) return b->fail(LBM_ERR_CUDA, "lbm_batch_set_tiling", e);
+    return LBM_OK;
+}
+
+// A batch whose tiling nobody has chosen (set_tiling, autotune) and whose waits nobody has
+// limited steps by one launch per step over tiles of 32 x 4 nodes, unless the persistent
+// kernel's default 128 x 16 tiles suit it: D2Q5 scalars, at least two tiles per CTA, and
+// lattices that fill the tiles' columns.  Microseconds per step, persistent : per step
+// (D2Q5): 4 lattices of 64^2 32.6 : 3.4, 16 of 96^2 32.7 : 8.0, 64 of 128^2 61.5 : 56.3
+// (fewer tiles than CTAs), 64 of sides 64 .. 512 332 : 308 and 256 of them 1385 : 1314 (a
+// sixth of the columns idle); 64 of 256^2 202 : 208 and 8 of 1024^2 407 : 409.  D2Q9: 64 of
+// 256^2 279 : 254, 8 of 1024^2 569 : 491.
+// Lattices too tall or large for the tiles' 32-bit offsets keep the persistent kernel.
+int choose_per_step(lbm_batch* b) {
+    std::vector<lbm::BatchTile> tiles;
+    long long strip_nodes = 0, tile_nodes = 0;
+    for (size_t c = 0; c < b->cases.size(); ++c) {
+        const lbm_handle* h = b->cases[c];
+        strip_nodes += (long long)((h->p.nx + b->tile_w - 1) / b->tile_w) * b->tile_w * h->p.ny;
+        tile_nodes += (long long)((h->p.nx + lbm::TILE_W - 1) / lbm::TILE_W) * lbm::TILE_W * h->p.ny;
+        if (h->L.pop_elems >= (1ULL << 31)) return LBM_OK;
+        for (int y = 0; y < h->p.ny; y += lbm::TILE_H)
+            for (int x = 0; x < h->p.nx; x += lbm::TILE_W)
+                tiles.push_back(lbm::BatchTile{(int)c, x, y, std::min(h->p.ny, y + lbm::TILE_H)});
+    }
+    if (b->q == 5 && b->ntiles >= 2 * b->grid && 100 * strip_nodes <= 103 * tile_nodes) return LBM_OK;
+    if ((long long)tiles.size() > std::min<long long>(b->tiles_cap, 0x7fffffff)) return LBM_OK;
+    cudaError_t e = cudaMemcpyAsync(b->d_tiles(), tiles.data(), tiles.size() * sizeof(lbm::BatchTile),
+                                    cudaMemcpyHostToDevice, b->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);  // the vector is pageable
+    if (e != cudaSuccess) return b->fail(LBM_ERR_CUDA, "lbm_batch_create: tiles", e);
+    b->per_step = true;
+    b->fine_tiles = (int)tiles.size();
     return LBM_OK;
 }
 
@@ -384,6 +459,7 @@ int lbm_batch_create(lbm_handle* const* cases, int32_t ncases, void* d_workspace
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->cases_ev, cudaEventDisableTiming);
     if (e == cudaSuccess) e = b->make_side_streams();
     rc = e == cudaSuccess ? build_tiling(b, 128, 16) : b->fail(LBM_ERR_CUDA, "lbm_batch_create: staging", e);
+    if (rc == LBM_OK) rc = choose_per_step(b);
     if (rc != LBM_OK) {
         snprintf(g_batch_error, sizeof(g_batch_error), "%s", b->err);
         lbm_batch_destroy(b);
@@ -418,6 +494,10 @@ int lbm_batch_step(lbm_batch* b, int64_t nsteps) {
     cudaError_t e = b->resync_cases();
     int64_t left = nsteps;
     const int G = lbm::detail::GRAPH_STEPS;
+    if (e == cudaSuccess && b->per_step) {
+        e = b->step_fine(left);
+        left = 0;
+    }
     if (e == cudaSuccess && left >= G) {
         if (!b->graph_tried) b->try_graph();
         while (e == cudaSuccess && left >= G) {
@@ -517,6 +597,11 @@ int lbm_batch_set_wait_limit(lbm_batch* b, int64_t spin_limit, int32_t hold_tile
     if (!b) return LBM_ERR_ARG;
     if (spin_limit < 1) return b->fail(LBM_ERR_ARG, "spin_limit must be >= 1");
     if (hold_tile < -1 || hold_tile >= b->ntiles) return b->fail(LBM_ERR_ARG, "hold_tile out of range");
+    if (b->per_step) {  // limited waits are those of the persistent kernel
+        lbm::detail::DeviceGuard dg(b->device);
+        const int rc = build_tiling(b, b->tile_w, b->tile_h);
+        if (rc != LBM_OK) return rc;
+    }
     b->spin_limit = spin_limit;
     b->hold_tile = hold_tile;
     b->drop_graph();

@@ -93,6 +93,33 @@ __global__ void __launch_bounds__(32 * NW, 20 / NW) batch_kernel(BatchArgs a) {
     }
 }
 
+// One step of every case, a tile of TILE_W x TILE_H nodes per CTA (tile_step): the steps
+// follow one another as launches instead of waiting for neighbours inside one.  A batch
+// that is small for the persistent kernel's tiles leaves SMs idle there and pays each
+// tile's rows one after another; here it takes a launch and one memory round trip per
+// step (measured at choose_per_step in lbm_batch.cu).
+template <int QS>
+__global__ void __launch_bounds__(TILE_W* TILE_H)
+    batch_tile_kernel(const BatchCase* __restrict__ cases, const BatchTile* __restrict__ tiles, unsigned t) {
+    constexpr int CASE_WORDS = (int)(sizeof(BatchCase) / sizeof(unsigned));
+    static_assert(sizeof(BatchCase) % sizeof(unsigned) == 0, "BatchCase is copied as words");
+    __shared__ BatchCase sc;
+    const BatchTile tl = tiles[blockIdx.x];
+    const unsigned* src = reinterpret_cast<const unsigned*>(cases + tl.c);
+    for (int w = threadIdx.x; w < CASE_WORDS; w += TILE_W * TILE_H) reinterpret_cast<unsigned*>(&sc)[w] = __ldg(src + w);
+    __syncthreads();
+    const int par = (int)((sc.cur0 + t) & 1u);
+    tile_step<float, float, QS>(static_cast<const float*>(sc.pop[par]), static_cast<float*>(sc.pop[par ^ 1]),
+                                static_cast<float*>(sc.prev), sc.g, sc.C, sc.flag, tl.x0, tl.ya);
+}
+
+template <int QS>
+cudaError_t launch_batch_tiles_impl(const BatchCase* cases, const BatchTile* tiles, int ntiles, int64_t t,
+                                    cudaStream_t s) {
+    batch_tile_kernel<QS><<<ntiles, TILE_W * TILE_H, 0, s>>>(cases, tiles, (unsigned)(t & 1));
+    return cudaGetLastError();
+}
+
 template <int QS, int NW>
 cudaError_t launch_batch_impl(const BatchArgs& a, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};

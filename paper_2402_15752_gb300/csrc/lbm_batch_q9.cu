@@ -20,4 +20,10 @@ LBM_BATCH_INSTANCE(4)
 
 #undef LBM_BATCH_INSTANCE
 
+template <>
+cudaError_t launch_batch_tiles<9>(const BatchCase* cases, const BatchTile* tiles, int ntiles, int64_t t,
+                                  cudaStream_t s) {
+    return launch_batch_tiles_impl<9>(cases, tiles, ntiles, t, s);
+}
+
 }  // namespace lbm

@@ -45,6 +45,8 @@ constexpr int STRIP_MIN_BLOCKS_16 = LBM_STRIP_MIN_BLOCKS_16;
 // FP64 arithmetic: 3 CTAs per SM (168 registers) keep it free of spills; its
 // speed is set by the FP64 pipe, not by memory
 constexpr int STRIP_MIN_BLOCKS_64 = 3;
+// Nodes of a CTA of the tile kernels (FP32 arithmetic)
+constexpr int TILE_W = 32, TILE_H = 4;
 // Blocks of the conserved-sum reduction (fixed, so the summation order is fixed).
 constexpr int RED_BLOCKS = 304;
 constexpr int RED_THREADS = 256;
@@ -211,6 +213,11 @@ struct BatchArgs {
     int hold_tile;            // fault injection: this tile never reports done (-1: none)
     int grid;                 // CTAs (all co-resident: cooperative launch)
 };
+
+// One step of every case in one launch of ntiles CTAs, tiles of TILE_W x TILE_H nodes;
+// t: steps completed since the case descriptors were written.
+template <int QS>
+cudaError_t launch_batch_tiles(const BatchCase* cases, const BatchTile* tiles, int ntiles, int64_t t, cudaStream_t s);
 
 // Tile widths of the batched kernel: 32 * NW columns, NW in {1, 2, 4}.
 template <int QS, int NW>
