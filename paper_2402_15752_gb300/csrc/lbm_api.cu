@@ -5,6 +5,7 @@
 #include "lbm.h"
 #include "lbm_handle.h"
 #include "lbm_internal.h"
+#include "lbm_kernels.cuh"
 
 #include <cmath>
 #include <cstdio>
@@ -107,16 +108,10 @@ lbm::Coeffs<R> coeffs_of(const lbm_params* p) {
     return C;
 }
 
-// two_over_W = 2 / W, taken once on the host: an FP64 division per node would
-// cost more than the kernel's memory traffic
 __global__ void sdf_to_fields_kernel(const double* __restrict__ sdf, double* phi, double* c1, double* c2,
                                      size_t n, double two_over_W, double c1t, double c2t) {
     for (size_t k = blockIdx.x * (size_t)blockDim.x + threadIdx.x; k < n; k += (size_t)gridDim.x * blockDim.x) {
-        const double a = sdf[k] * two_over_W;
-        // Eq. (2).  tanh saturates: for |a| >= 20, 1 - |tanh a| < 1e-17, below half
-        // the spacing of doubles under 1, so the rounded profile is exactly 0 or 1
-        // there, and only the interface band pays for the FP64 tanh
-        const double ph = fabs(a) >= 20.0 ? (a > 0.0 ? 1.0 : 0.0) : 0.5 + 0.5 * tanh(a);
+        const double ph = lbm::sdf_phi(sdf[k], two_over_W);
         phi[k] = ph;
         c1[k] = c1t * ph;
         c2[k] = c2t * (1.0 - ph);
@@ -274,13 +269,16 @@ int lbm_create(const lbm_params* params, void* d_workspace, size_t workspace_byt
     return LBM_OK;
 }
 
-static int init_common(lbm_handle* h, const double* phi, const double* c1, const double* c2,
-                       const double* ux = nullptr, const double* uy = nullptr, const double* p = nullptr) {
-    const lbm::InitFields in{phi, ux, uy, p, c1, c2};
+static int init_with(lbm_handle* h, const lbm::InitFields& in) {
     const cudaError_t e = h->init_on(in, h->stream);
     if (e != cudaSuccess) return h->fail(LBM_ERR_CUDA, "init kernel", e);
     h->restarted();
     return LBM_OK;
+}
+
+static int init_common(lbm_handle* h, const double* phi, const double* c1, const double* c2,
+                       const double* ux = nullptr, const double* uy = nullptr, const double* p = nullptr) {
+    return init_with(h, lbm::InitFields{phi, ux, uy, p, c1, c2});
 }
 
 // Device address of a host buffer that the GPU can read and write in place
@@ -314,6 +312,16 @@ int lbm_init(lbm_handle* h, const double* sdf, int32_t sdf_on_device, double c1_
             src = phi;
         }
     }
+    if (h->L.elem != 2) {  // one pass: the initialisation evaluates the profile itself
+        if (e != cudaSuccess) return h->fail(LBM_ERR_CUDA, "lbm_init", e);
+        lbm::InitFields in{src, nullptr, nullptr, nullptr, nullptr, nullptr};
+        in.sdf = true;
+        in.two_over_W = 2.0 / h->p.W;
+        in.c1t = c1_tilde;
+        in.c2t = c2_tilde;
+        return init_with(h, in);
+    }
+    // 16-bit storage: a node's populations are relative to its neighbours' fields
     if (e == cudaSuccess) e = lbm::launch_sdf_to_fields(src, phi, c1, c2, n, h->p.W, c1_tilde, c2_tilde, h->stream);
     if (e != cudaSuccess) return h->fail(LBM_ERR_CUDA, "lbm_init", e);
     return init_common(h, phi, c1, c2);

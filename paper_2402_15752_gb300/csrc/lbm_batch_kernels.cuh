@@ -116,8 +116,7 @@ __global__ void __launch_bounds__(TILE_W* TILE_H)
 template <int QS>
 cudaError_t launch_batch_tiles_impl(const BatchCase* cases, const BatchTile* tiles, int ntiles, int64_t t,
                                     cudaStream_t s) {
-    batch_tile_kernel<QS><<<ntiles, TILE_W * TILE_H, 0, s>>>(cases, tiles, (unsigned)(t & 1));
-    return cudaGetLastError();
+    return launch_overlapped(batch_tile_kernel<QS>, dim3(ntiles), TILE_W * TILE_H, s, cases, tiles, (unsigned)(t & 1));
 }
 
 template <int QS, int NW>

@@ -159,6 +159,10 @@ cudaError_t launch_variant(const void* src, void* dst, void* prev, const Geometr
 // may be NULL (zero).
 struct InitFields {
     const double *phi, *ux, *uy, *p, *c1, *c2;
+    // sdf: phi holds signed distances (Eq. 2 with 2 / W), c1 = c1t phi, c2 = c2t (1 - phi),
+    // c1 and c2 unused (FP32 and FP64 storage)
+    bool sdf = false;
+    double two_over_W = 0.0, c1t = 0.0, c2t = 0.0;
 };
 
 // Initial populations at the equilibria of the given fields, written
