@@ -269,8 +269,12 @@ void lbm_destroy(lbm_handle* h);
 /*
  * Batched runner.  Many independent lattices of uneven sizes (each an lbm_handle
  * with its own parameters and workspace) advanced together by one persistent
- * kernel: each lattice is cut into tiles of tile_w x tile_h nodes, the launch's
- * CTAs (all co-resident: a cooperative launch) own the tiles round-robin, and a
+ * kernel, or by one launch per step: a batch whose tiling nobody has chosen
+ * (lbm_batch_set_tiling, lbm_batch_autotune) and whose waits nobody has limited
+ * (lbm_batch_set_wait_limit) steps by launches over tiles of 32 x 4 nodes where that is
+ * the faster.  The persistent kernel: each lattice is cut into tiles of tile_w x
+ * tile_h nodes, the launch's CTAs (all co-resident: a cooperative launch) own the
+ * tiles round-robin, and a
  * tile waits only for the tiles of the same lattice whose nodes it reads or that
  * read its nodes (usually the 8 around it) to finish the previous step (per-tile
  * step counters), never for the whole grid.  Full runs of

@@ -161,6 +161,8 @@ static int choose_strip_height(const lbm_handle* h) {
 
 // Whether the step runs tiles (tile_kernel, tile64_kernel) instead of strips.  Times
 // are microseconds per step, strips against tiles, on square periodic lattices:
+// (The tiles' launches overlap since: 64^2 takes 2.75 in FP32, 3.4 in bfloat16, 12.7 in
+// FP64; the lines stayed.)
 // * FP64 always: 64^2 82 : 14, 512^2 275 : 165, 1024^2 938 : 622 (D2Q5).  Tiles of 8 x 4
 //   nodes while they leave SMs idle or nearly so (64^2: 13.9 against 15.2 with 16 x 8),
 //   else 16 x 8, whose ring is smaller (128^2: 15.3 against 16.2, 512^2: 165 : 174).

@@ -2,7 +2,8 @@
 // FP32 lattices, each an lbm_handle of its own, advanced together by the
 // persistent batched kernel (lbm_batch_kernels.cuh) in one cooperative launch
 // per call -- or per 32 steps, replayed from a captured CUDA graph -- with the
-// tile shape chosen by timing candidates (lbm_batch_autotune).
+// tile shape chosen by timing candidates (lbm_batch_autotune); or, by default where
+// that is the faster (choose_per_step), by one launch of small tiles per step.
 #include "lbm.h"
 #include "lbm_handle.h"
 #include "lbm_internal.h"
@@ -395,10 +396,10 @@ int build_tiling(lbm_batch* b, int tile_w, int tile_h) {
 // limited steps by one launch per step over tiles of 32 x 4 nodes, unless the persistent
 // kernel's default 128 x 16 tiles suit it: D2Q5 scalars, at least two tiles per CTA, and
 // lattices that fill the tiles' columns.  Microseconds per step, persistent : per step
-// (D2Q5): 4 lattices of 64^2 32.6 : 3.4, 16 of 96^2 32.7 : 8.0, 64 of 128^2 61.5 : 56.3
-// (fewer tiles than CTAs), 64 of sides 64 .. 512 332 : 308 and 256 of them 1385 : 1314 (a
-// sixth of the columns idle); 64 of 256^2 202 : 208 and 8 of 1024^2 407 : 409.  D2Q9: 64 of
-// 256^2 279 : 254, 8 of 1024^2 569 : 491.
+// (D2Q5): 4 lattices of 64^2 32.3 : 2.6, 16 of 96^2 32.7 : 7.3, 64 of 128^2 61.5 : 55.3
+// (fewer tiles than CTAs), 64 of sides 64 .. 512 332 : 307 and 256 of them 1383 : 1313 (a
+// sixth of the columns idle); 64 of 256^2 202 : 208 and 8 of 1024^2 407 : 409 before the
+// steps' launches overlapped.  D2Q9: 64 of 256^2 279 : 254, 8 of 1024^2 567 : 490.
 // Lattices too tall or large for the tiles' 32-bit offsets keep the persistent kernel.
 int choose_per_step(lbm_batch* b) {
     std::vector<lbm::BatchTile> tiles;
