@@ -107,11 +107,12 @@ __global__ void __launch_bounds__(256)
 // GB300) bounds a version that forms every square in double: 208 us at 16 x 256 x
 // 256 pixels, over the 16 channels of which 5 are used.  Here the difference is
 // split exactly into two floats, s + e = pred - target (Knuth's two-sum), its
-// square into h + l (a fused multiply-add gives the product's rounding error), and
-// the pixel's squares are added as such pairs; only the pixel's sum is converted
-// and added in double.  The pairs carry 2^-46 of a pixel's sum, far below the
-// rounding of the double total over the pixels.  Squares that would leave the
-// float range take the double form.
+// square into h + l + p + q + e^2 (a fused multiply-add gives a product's rounding
+// error), and the pixel's squares are added as triples of floats H + M + L; only
+// the pixel's sum is converted and added in double.  L is 2^-48 of the sum and
+// carries 24 bits, so a pixel's sum is exact to better than 2^-60, where adding the
+// squares in double rounded once per channel.  (As pairs, without L: 2^-46.)
+// Squares that would leave the float range take the double form.
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
     s = __fadd_rn(a, b);
     const float bb = __fsub_rn(s, a);
@@ -159,7 +160,7 @@ __global__ void __launch_bounds__(256)
     };
     auto pixel = [&](long long p, const float (&x)[4 * NV], const float (&y)[4 * NV]) {
         float g[16] = {};
-        float H = 0.0f, L = 0.0f;
+        float H = 0.0f, M = 0.0f, L = 0.0f;
         bool odd = false;  // a difference whose square leaves the float range
 #pragma unroll
         for (int c = 0; c < 4 * NV; ++c) {
@@ -168,20 +169,22 @@ __global__ void __launch_bounds__(256)
             two_sum(x[c], -y[c], s, e);
             const float m = fabsf(s);
             odd |= !(m == 0.0f || (m > 1e-14f && m < 1e18f));  // also NaN
-            const float h = __fmul_rn(s, s);
-            // the product's error, and the cross term of the split
-            const float l = __fadd_rn(__fmaf_rn(s, s, -h), __fmul_rn(2.0f * s, e));
-            float z, r;
-            two_sum(H, h, z, r);
-            H = z;
-            L = __fadd_rn(L, __fadd_rn(r, l));
+            // (s + e)^2 = h + l + p + q + e^2
+            const float h = __fmul_rn(s, s), l = __fmaf_rn(s, s, -h);
+            const float s2 = 2.0f * s, p = __fmul_rn(s2, e), q = __fmaf_rn(s2, e, -p);
+            float r0, r1, r2, r3;
+            two_sum(H, h, H, r0);
+            two_sum(M, r0, M, r1);
+            two_sum(M, l, M, r2);
+            two_sum(M, p, M, r3);
+            L = __fadd_rn(L, __fadd_rn(__fadd_rn(__fadd_rn(r1, r2), r3), __fmaf_rn(e, e, q)));
             g[c] = __fmaf_rn(khi, s, __fmaf_rn(khi, e, __fmul_rn(klo, s)));
         }
         if (odd) {
             a += pixel_in_double(pred + p * 16, target + p * 16, U, 2.0 * inv, dpred ? dpred + p * 16 : nullptr);
             return;
         }
-        a += (double)H + (double)L;
+        a += (double)H + ((double)M + (double)L);
         if (!dpred) return;
         if constexpr (VEC) {
             uint32_t out[8];
