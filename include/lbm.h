@@ -300,18 +300,25 @@ typedef struct lbm_batch lbm_batch;
 size_t lbm_batch_workspace_bytes(lbm_handle* const* cases, int32_t ncases);
 
 /* Build a batch over ncases handles (the array is copied; the handles stay the
- * caller's) with a caller-owned, 256-byte aligned device workspace.  The initial
- * tiling is 128 x 16.  Synchronises the stream. */
+ * caller's) with a caller-owned, 256-byte aligned device workspace.  It steps by one
+ * launch per step where that is the faster (lbm_batch_per_step), else by the persistent
+ * kernel, whose initial tiling is 128 x 16.  Synchronises the stream. */
 int lbm_batch_create(lbm_handle* const* cases, int32_t ncases, void* d_workspace,
                      size_t workspace_bytes, lbm_batch** out);
 
-/* Tile shape: tile_w in {32, 64, 128} columns, tile_h >= 4 rows.  Rebuilds the
- * tile tables and restarts the step counters; synchronises. */
+/* Step by the persistent kernel in tiles of tile_w in {32, 64, 128} columns and tile_h
+ * >= 4 rows.  Rebuilds the tile tables and restarts the step counters; synchronises. */
 int lbm_batch_set_tiling(lbm_batch* b, int32_t tile_w, int32_t tile_h);
 
-/* Current tile shape, tile count and CTAs per launch (any pointer may be NULL). */
+/* The persistent kernel's tile shape, tile count and CTAs per launch (any pointer may be
+ * NULL).  While lbm_batch_per_step is 1 the batch does not run them: its launches have one
+ * CTA per tile of 32 x 4 nodes. */
 int lbm_batch_tiling(const lbm_batch* b, int32_t* tile_w, int32_t* tile_h, int32_t* ntiles,
                      int32_t* grid);
+
+/* 1: the batch steps by one launch per step; 0: by the persistent kernel; negative: an
+ * error code. */
+int lbm_batch_per_step(const lbm_batch* b);
 
 /* Advance every case by nsteps >= 0 time steps (asynchronous on the stream). */
 int lbm_batch_step(lbm_batch* b, int64_t nsteps);

@@ -1,5 +1,6 @@
 """Batched runner: many independent FP32 lattices (Simulation objects) advanced
-together by the library's persistent batched kernel (lbm_batch_* in lbm.h).
+together by the library (lbm_batch_* in lbm.h): by a persistent kernel, or by one launch
+per step over small tiles.
 
 Argument marshalling only: the tile tables, the launch and the autotuner's
 timing loop are in the library.  The autotuner's choice can be cached in a
@@ -111,9 +112,12 @@ class Batch:
         _check(self.L, self._b, self.L.lbm_batch_set_tiling(self._b, int(tile_w), int(tile_h)))
 
     def tiling(self) -> dict:
+        """The persistent kernel's tiles, and whether the batch steps by one launch per
+        step over tiles of 32 x 4 nodes instead (per_step)."""
         v = [ctypes.c_int32() for _ in range(4)]
         _check(self.L, self._b, self.L.lbm_batch_tiling(self._b, *[ctypes.byref(x) for x in v]))
-        return dict(tile_w=v[0].value, tile_h=v[1].value, tiles=v[2].value, ctas=v[3].value)
+        return dict(tile_w=v[0].value, tile_h=v[1].value, tiles=v[2].value, ctas=v[3].value,
+                    per_step=self.L.lbm_batch_per_step(self._b) == 1)
 
     def set_wait_limit(self, spin_limit: int, hold_tile: int = -1):
         _check(self.L, self._b, self.L.lbm_batch_set_wait_limit(self._b, int(spin_limit), int(hold_tile)))

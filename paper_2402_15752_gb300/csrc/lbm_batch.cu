@@ -485,6 +485,8 @@ int lbm_batch_tiling(const lbm_batch* b, int32_t* tile_w, int32_t* tile_h, int32
     return LBM_OK;
 }
 
+int lbm_batch_per_step(const lbm_batch* b) { return b ? (int)b->per_step : LBM_ERR_ARG; }
+
 int lbm_batch_step(lbm_batch* b, int64_t nsteps) {
     const lbm::NvtxRange range("lbm_batch_step");
     if (!b) return LBM_ERR_ARG;

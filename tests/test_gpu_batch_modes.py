@@ -1,0 +1,36 @@
+"""The two ways a batch steps, one launch per step and the persistent kernel: which one
+runs, the way from one to the other, and the same fields as lattices stepped alone."""
+import ctypes
+
+import pytest
+
+from paper_2402_15752_gb300 import Batch, Simulation
+from paper_2402_15752_gb300 import workloads as wl
+
+from test_gpu_batch import _assert_same, _cases, _sims
+
+pytestmark = pytest.mark.gpu
+
+
+def _squares(sides, **over):
+    return [wl.droplet64(nx=n, ny=n, R=0.3 * n, **over) for n in sides]
+
+
+@pytest.mark.parametrize("sides,per_step", [([64] * 4, True), ([768] * 8, False)])
+def test_the_batch_says_how_it_steps(sides, per_step):
+    # 8 x 768^2: 2304 tiles of 128 x 16, two for each of 7 CTAs per SM, no idle column
+    cases = _squares(sides)
+    sims, alone = _sims(cases), _sims(cases)
+    b = Batch(sims)
+    t = b.tiling()
+    assert t["per_step"] is per_step
+    assert (t["tile_w"], t["tile_h"]) == (128, 16)
+    b.step(5)
+    b.sync()
+    for s in alone:
+        s.step(5)
+    _assert_same(sims, alone, label="default mode")
+    b.set_tiling(64, 16)
+    assert not b.tiling()["per_step"]
+    b.close()
+    assert b.L.lbm_batch_per_step(ctypes.c_void_p()) == -1
