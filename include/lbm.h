@@ -337,7 +337,9 @@ int lbm_batch_autotune(lbm_batch* b, int32_t steps_per_trial, double* table, int
 
 /* Fault injection for tests of the bounded waits: polls per wait before it gives
  * up (default 2^21, about a second) and a tile whose completion is never
- * published (-1: none). */
+ * published (-1: none).  The waits are the persistent kernel's: a batch that steps by one
+ * launch per step goes over to it (restarting the step counters), and back with
+ * the defaults. */
 int lbm_batch_set_wait_limit(lbm_batch* b, int64_t spin_limit, int32_t hold_tile);
 
 /* Restart every case at the equilibria of its six macroscopic fields, as

@@ -106,6 +106,7 @@ struct lbm_batch {
     // one launch per step over tiles of TILE_W x TILE_H (table in d_tiles) instead of the
     // persistent kernel; its 32-step graphs by the parity of the first step
     bool per_step = false;
+    bool want_per_step = false;  // ... where no limit of the waits asks for the persistent kernel
     int fine_tiles = 0;
     cudaGraphExec_t step_graph[2] = {};
     // pinned staging of the case descriptors; the event marks the end of the
@@ -392,6 +393,30 @@ int build_tiling(lbm_batch* b, int tile_w, int tile_h) {
     return LBM_OK;
 }
 
+// The 32 x 4 tiles of every case; false for lattices too tall or large for their 32-bit
+// offsets or for the tile table.
+bool fine_tiling(const lbm_batch* b, std::vector<lbm::BatchTile>& tiles) {
+    for (size_t c = 0; c < b->cases.size(); ++c) {
+        const lbm_handle* h = b->cases[c];
+        if (h->L.pop_elems >= (1ULL << 31)) return false;
+        for (int y = 0; y < h->p.ny; y += lbm::TILE_H)
+            for (int x = 0; x < h->p.nx; x += lbm::TILE_W)
+                tiles.push_back(lbm::BatchTile{(int)c, x, y, std::min(h->p.ny, y + lbm::TILE_H)});
+    }
+    return (long long)tiles.size() <= std::min<long long>(b->tiles_cap, 0x7fffffff);
+}
+
+// Step by one launch per step from here on (the tile table is rewritten; synchronises).
+int start_per_step(lbm_batch* b, const std::vector<lbm::BatchTile>& tiles) {
+    cudaError_t e = cudaMemcpyAsync(b->d_tiles(), tiles.data(), tiles.size() * sizeof(lbm::BatchTile),
+                                    cudaMemcpyHostToDevice, b->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);  // the vector is pageable
+    if (e != cudaSuccess) return b->fail(LBM_ERR_CUDA, "batched runner: tiles", e);
+    b->per_step = true;
+    b->fine_tiles = (int)tiles.size();
+    return LBM_OK;
+}
+
 // A batch whose tiling nobody has chosen (set_tiling, autotune) and whose waits nobody has
 // limited steps by one launch per step over tiles of 32 x 4 nodes, unless the persistent
 // kernel's default 128 x 16 tiles suit it: D2Q5 scalars, at least two tiles per CTA, and
@@ -400,28 +425,17 @@ int build_tiling(lbm_batch* b, int tile_w, int tile_h) {
 // (fewer tiles than CTAs), 64 of sides 64 .. 512 332 : 307 and 256 of them 1383 : 1313 (a
 // sixth of the columns idle); 64 of 256^2 202 : 208 and 8 of 1024^2 407 : 409 before the
 // steps' launches overlapped.  D2Q9: 64 of 256^2 279 : 254, 8 of 1024^2 567 : 490.
-// Lattices too tall or large for the tiles' 32-bit offsets keep the persistent kernel.
 int choose_per_step(lbm_batch* b) {
     std::vector<lbm::BatchTile> tiles;
+    if (!fine_tiling(b, tiles)) return LBM_OK;
     long long strip_nodes = 0, tile_nodes = 0;
-    for (size_t c = 0; c < b->cases.size(); ++c) {
-        const lbm_handle* h = b->cases[c];
+    for (const lbm_handle* h : b->cases) {
         strip_nodes += (long long)((h->p.nx + b->tile_w - 1) / b->tile_w) * b->tile_w * h->p.ny;
         tile_nodes += (long long)((h->p.nx + lbm::TILE_W - 1) / lbm::TILE_W) * lbm::TILE_W * h->p.ny;
-        if (h->L.pop_elems >= (1ULL << 31)) return LBM_OK;
-        for (int y = 0; y < h->p.ny; y += lbm::TILE_H)
-            for (int x = 0; x < h->p.nx; x += lbm::TILE_W)
-                tiles.push_back(lbm::BatchTile{(int)c, x, y, std::min(h->p.ny, y + lbm::TILE_H)});
     }
     if (b->q == 5 && b->ntiles >= 2 * b->grid && 100 * strip_nodes <= 103 * tile_nodes) return LBM_OK;
-    if ((long long)tiles.size() > std::min<long long>(b->tiles_cap, 0x7fffffff)) return LBM_OK;
-    cudaError_t e = cudaMemcpyAsync(b->d_tiles(), tiles.data(), tiles.size() * sizeof(lbm::BatchTile),
-                                    cudaMemcpyHostToDevice, b->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);  // the vector is pageable
-    if (e != cudaSuccess) return b->fail(LBM_ERR_CUDA, "lbm_batch_create: tiles", e);
-    b->per_step = true;
-    b->fine_tiles = (int)tiles.size();
-    return LBM_OK;
+    b->want_per_step = true;
+    return start_per_step(b, tiles);
 }
 
 }  // namespace
@@ -473,7 +487,9 @@ int lbm_batch_create(lbm_handle* const* cases, int32_t ncases, void* d_workspace
 int lbm_batch_set_tiling(lbm_batch* b, int32_t tile_w, int32_t tile_h) {
     if (!b) return LBM_ERR_ARG;
     lbm::detail::DeviceGuard dg(b->device);
-    return build_tiling(b, tile_w, tile_h);
+    const int rc = build_tiling(b, tile_w, tile_h);
+    if (rc == LBM_OK) b->want_per_step = false;
+    return rc;
 }
 
 int lbm_batch_tiling(const lbm_batch* b, int32_t* tile_w, int32_t* tile_h, int32_t* ntiles, int32_t* grid) {
@@ -593,6 +609,7 @@ int lbm_batch_autotune(lbm_batch* b, int32_t steps_per_trial, double* table, int
     cudaEventDestroy(e1);
     if (rows_written) *rows_written = rows;
     if (rc != LBM_OK) return rc;
+    b->want_per_step = false;
     return build_tiling(b, best_w, best_h);
 }
 
@@ -600,11 +617,17 @@ int lbm_batch_set_wait_limit(lbm_batch* b, int64_t spin_limit, int32_t hold_tile
     if (!b) return LBM_ERR_ARG;
     if (spin_limit < 1) return b->fail(LBM_ERR_ARG, "spin_limit must be >= 1");
     if (hold_tile < -1 || hold_tile >= b->ntiles) return b->fail(LBM_ERR_ARG, "hold_tile out of range");
-    if (b->per_step) {  // limited waits are those of the persistent kernel
-        lbm::detail::DeviceGuard dg(b->device);
-        const int rc = build_tiling(b, b->tile_w, b->tile_h);
-        if (rc != LBM_OK) return rc;
+    // limited waits are those of the persistent kernel; the defaults give back the launches
+    // per step of a batch that had them
+    lbm::detail::DeviceGuard dg(b->device);
+    int rc = LBM_OK;
+    if (spin_limit != DEFAULT_SPIN_LIMIT || hold_tile != -1) {
+        if (b->per_step) rc = build_tiling(b, b->tile_w, b->tile_h);
+    } else if (b->want_per_step && !b->per_step) {
+        std::vector<lbm::BatchTile> tiles;
+        if (fine_tiling(b, tiles)) rc = start_per_step(b, tiles);
     }
+    if (rc != LBM_OK) return rc;
     b->spin_limit = spin_limit;
     b->hold_tile = hold_tile;
     b->drop_graph();

@@ -34,3 +34,29 @@ def test_the_batch_says_how_it_steps(sides, per_step):
     assert not b.tiling()["per_step"]
     b.close()
     assert b.L.lbm_batch_per_step(ctypes.c_void_p()) == -1
+
+
+def test_default_waits_leave_the_launches_per_step():
+    cases = _cases()
+    sims, alone = _sims(cases), _sims(cases)
+    b = Batch(sims)
+    assert b.tiling()["per_step"]
+    b.step(3)
+    b.set_wait_limit(1 << 21, -1)  # the defaults
+    assert b.tiling()["per_step"]
+    b.step(4)
+    b.set_wait_limit(1 << 20, -1)  # 7 steps in: a limit, and back after an odd number of steps
+    assert not b.tiling()["per_step"]
+    b.step(35)
+    b.set_wait_limit(1 << 21, -1)
+    assert b.tiling()["per_step"]
+    b.step(33)
+    b.set_tiling(32, 8)  # the persistent kernel by choice: the defaults leave it
+    b.set_wait_limit(1 << 21, -1)
+    assert not b.tiling()["per_step"]
+    b.step(6)
+    b.sync()
+    for s in alone:
+        s.step(3 + 4 + 35 + 33 + 6)
+    _assert_same(sims, alone, label="modes in turn")
+    b.close()
