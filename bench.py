@@ -446,7 +446,7 @@ def secondary(dev):
         ms = timed_steps(b.step, sims[0].stream, 200, 5)
         b.sync()
         out["batched256_fp32"] = entry(sum(w.cells for w in cases), 200, ms, 264, cases=len(cases),
-                                       tiling={k: tune[k] for k in ("tile_w", "tile_h")})
+                                       tiling={k: tune[k] for k in ("tile_w", "tile_h", "per_step")})
     except Exception as e:
         out["batched256_fp32"] = {"failed": str(e)[:200]}
     finally:
@@ -458,8 +458,8 @@ def secondary(dev):
 
 
 def run_batched(args, rank, world, local):
-    """256 independent droplets of uneven sizes in the persistent batched kernel,
-    tile shape picked by the autotuner; compared with stepping every case with its
+    """256 independent droplets of uneven sizes in the batched runner, its launches per
+    step or the persistent kernel's tile shape picked by the autotuner; compared with stepping every case with its
     own launches (graph-replayed lbm_step), one case after another."""
     import numpy as np
     import torch
@@ -576,7 +576,7 @@ def run_batched(args, rank, world, local):
             "config": {"workload": "batched256", "cases": len(cases), "cells": cells,
                        "sides": "64..512 step 32", "bc": "periodic", "scalar_q": 5,
                        "precision": "fp32", "l2": "state larger than L2 (no flush)",
-                       "tiling": {k: tune[k] for k in ("tile_w", "tile_h", "tiles", "ctas")},
+                       "tiling": {k: tune[k] for k in ("tile_w", "tile_h", "tiles", "ctas", "per_step")},
                        "per_case_launches_mlups": per_case, "per_case_steps": per_steps,
                        "parallelism": "replicas" if world > 1 else "single"},
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
@@ -584,7 +584,7 @@ def run_batched(args, rank, world, local):
                          "peak_source": peak_kind, "bytes_per_cell": bytes_per_cell},
             "cpu_baseline": cpu,
             "e2e": e2e,
-            "gpu_launches": graphs + (1 if rest else 0),
+            "gpu_launches": args.steps if tune["per_step"] else graphs + (1 if rest else 0),
             "clocks": clocks,
         }
         print(json.dumps(line), flush=True)

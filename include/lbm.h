@@ -269,10 +269,10 @@ void lbm_destroy(lbm_handle* h);
 /*
  * Batched runner.  Many independent lattices of uneven sizes (each an lbm_handle
  * with its own parameters and workspace) advanced together by one persistent
- * kernel, or by one launch per step: a batch whose tiling nobody has chosen
- * (lbm_batch_set_tiling, lbm_batch_autotune) and whose waits nobody has limited
- * (lbm_batch_set_wait_limit) steps by launches over tiles of 32 x 4 nodes where that is
- * the faster.  The persistent kernel: each lattice is cut into tiles of tile_w x
+ * kernel, or by one launch per step: a batch for which nobody has chosen otherwise
+ * (lbm_batch_set_per_step, lbm_batch_set_tiling, lbm_batch_autotune) and whose waits
+ * nobody has limited (lbm_batch_set_wait_limit) steps by launches over tiles of 32 x 4
+ * nodes where that is the faster.  The persistent kernel: each lattice is cut into tiles of tile_w x
  * tile_h nodes, the launch's CTAs (all co-resident: a cooperative launch) own the
  * tiles round-robin, and a
  * tile waits only for the tiles of the same lattice whose nodes it reads or that
@@ -320,6 +320,11 @@ int lbm_batch_tiling(const lbm_batch* b, int32_t* tile_w, int32_t* tile_h, int32
  * error code. */
 int lbm_batch_per_step(const lbm_batch* b);
 
+/* Choose: 1 the launches per step (from the defaults of lbm_batch_set_wait_limit on, if
+ * the waits are limited), 0 the persistent kernel with the tiles of lbm_batch_tiling.
+ * LBM_ERR_ARG for 1 if a lattice has 2^31 or more stored populations.  Synchronises. */
+int lbm_batch_set_per_step(lbm_batch* b, int32_t on);
+
 /* Advance every case by nsteps >= 0 time steps (asynchronous on the stream). */
 int lbm_batch_step(lbm_batch* b, int64_t nsteps);
 
@@ -327,11 +332,14 @@ int lbm_batch_step(lbm_batch* b, int64_t nsteps);
  * LBM_ERR_NONFINITE, else LBM_OK. */
 int lbm_batch_sync(lbm_batch* b);
 
-/* Time every candidate tiling (tile_w 32, 64, 128 x tile_h 8, 16, 32, 64) over
- * steps_per_trial steps (after 2 untimed ones) and keep the fastest.  The trial
- * steps are real steps of every case (every tiling computes the same update), so
- * the cases advance by 12 * (steps_per_trial + 2) steps.  table (optional) receives
- * up to table_rows rows of {tile_w, tile_h, ms per step, tiles, CTAs}. */
+/* Time every candidate tiling of the persistent kernel (tile_w 32, 64, 128 x tile_h 8, 16,
+ * 32, 64) over steps_per_trial steps, and the launches per step over 10 (unless a
+ * lattice is too large for them or the waits are limited), and keep the fastest:
+ * lbm_batch_tiling then reports the fastest tiling, lbm_batch_per_step whether the
+ * launches per step were as fast.  The trial steps are real steps of every case (every
+ * mode computes the same update), so the cases advance by 12 * (steps_per_trial + 2)
+ * steps, the untimed ones among them.  table (optional) receives up to table_rows
+ * rows of {tile_w, tile_h, ms per step, tiles, CTAs}, one per tiling. */
 int lbm_batch_autotune(lbm_batch* b, int32_t steps_per_trial, double* table, int32_t table_rows,
                        int32_t* rows_written);
 

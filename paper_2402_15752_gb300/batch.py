@@ -119,6 +119,9 @@ class Batch:
         return dict(tile_w=v[0].value, tile_h=v[1].value, tiles=v[2].value, ctas=v[3].value,
                     per_step=self.L.lbm_batch_per_step(self._b) == 1)
 
+    def set_per_step(self, on: bool = True):
+        _check(self.L, self._b, self.L.lbm_batch_set_per_step(self._b, int(bool(on))))
+
     def set_wait_limit(self, spin_limit: int, hold_tile: int = -1):
         _check(self.L, self._b, self.L.lbm_batch_set_wait_limit(self._b, int(spin_limit), int(hold_tile)))
 
@@ -131,16 +134,22 @@ class Batch:
         return hashlib.sha256(raw.encode()).hexdigest()[:16]
 
     def autotune(self, steps_per_trial: int = 20, cache: str | None = None) -> dict:
-        """Pick the fastest tiling by timing each candidate (the trial steps are
+        """Pick the fastest tiling of the persistent kernel, or the launches per step
+        where they are as fast (per_step), by timing each (the trial steps are
         real steps of every case).  With `cache`, a JSON file, a choice stored for
         the same signature is applied without timing, and a new one is stored."""
         key = self.signature()
+        mode = key + ".per_step"
         if cache and os.path.exists(cache):
             with open(cache) as f:
                 known = json.load(f)
             if key in known:
+                # a choice stored without its mode leaves the mode as it is
+                per_step = bool(known.get(mode, self.tiling()["per_step"]))
                 self.set_tiling(known[key]["tile_w"], known[key]["tile_h"])
-                return dict(known[key], cached=True)
+                if per_step:
+                    self.set_per_step(True)
+                return dict(known[key], per_step=per_step, cached=True)
         rows = 12
         table = (ctypes.c_double * (5 * rows))()
         written = ctypes.c_int32()
@@ -156,6 +165,7 @@ class Batch:
                 with open(cache) as f:
                     known = json.load(f)
             known[key] = {"tile_w": choice["tile_w"], "tile_h": choice["tile_h"]}
+            known[mode] = choice["per_step"]
             with open(cache, "w") as f:
                 json.dump(known, f, indent=1, sort_keys=True)
         return choice

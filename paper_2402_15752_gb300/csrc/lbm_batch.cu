@@ -160,6 +160,8 @@ struct lbm_batch {
         return e;
     }
 
+    bool limited_waits() const { return spin_limit != DEFAULT_SPIN_LIMIT || hold_tile != -1; }
+
     lbm::BatchCase* d_cases() const { return reinterpret_cast<lbm::BatchCase*>(ws + L.off_cases); }
     lbm::BatchTile* d_tiles() const { return reinterpret_cast<lbm::BatchTile*>(ws + L.off_tiles); }
     int* d_nbr() const { return reinterpret_cast<int*>(ws + L.off_nbr); }
@@ -246,6 +248,24 @@ struct lbm_batch {
                       : lbm::launch_batch_tiles<9>(d_cases(), d_tiles(), fine_tiles, t, s);
     }
 
+    // A graph of n steps from step t on
+    cudaError_t capture_fine(int64_t t, int n, cudaGraphExec_t* exec) {
+        cudaStream_t cap = nullptr;
+        cudaGraph_t g = nullptr;
+        cudaError_t e = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking);
+        if (e == cudaSuccess) e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
+        if (e == cudaSuccess) {
+            cudaError_t le = cudaSuccess;
+            for (int k = 0; k < n && le == cudaSuccess; ++k) le = launch_fine(t + k, cap);
+            e = cudaStreamEndCapture(cap, &g);
+            if (le != cudaSuccess) e = le;
+        }
+        if (e == cudaSuccess) e = cudaGraphInstantiate(exec, g, 0);
+        if (g) cudaGraphDestroy(g);
+        if (cap) cudaStreamDestroy(cap);
+        return e;
+    }
+
     // nsteps steps as launches, full runs of GRAPH_STEPS from a captured graph
     cudaError_t step_fine(int64_t nsteps) {
         constexpr int G = lbm::detail::GRAPH_STEPS;
@@ -253,21 +273,7 @@ struct lbm_batch {
         int64_t done = 0;
         for (; e == cudaSuccess && nsteps - done >= G; done += G) {
             cudaGraphExec_t& exec = step_graph[(steps + done) & 1];
-            if (!exec) {
-                cudaStream_t cap = nullptr;
-                cudaGraph_t g = nullptr;
-                e = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking);
-                if (e == cudaSuccess) e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
-                if (e == cudaSuccess) {
-                    cudaError_t le = cudaSuccess;
-                    for (int k = 0; k < G && le == cudaSuccess; ++k) le = launch_fine(steps + done + k, cap);
-                    e = cudaStreamEndCapture(cap, &g);
-                    if (le != cudaSuccess) e = le;
-                }
-                if (e == cudaSuccess) e = cudaGraphInstantiate(&exec, g, 0);
-                if (g) cudaGraphDestroy(g);
-                if (cap) cudaStreamDestroy(cap);
-            }
+            if (!exec) e = capture_fine(steps + done, G, &exec);
             if (e == cudaSuccess) e = cudaGraphLaunch(exec, stream);
         }
         for (; e == cudaSuccess && done < nsteps; ++done) e = launch_fine(steps + done, stream);
@@ -566,33 +572,55 @@ int lbm_batch_autotune(lbm_batch* b, int32_t steps_per_trial, double* table, int
     lbm::detail::DeviceGuard dg(b->device);
     static const int widths[] = {32, 64, 128};
     static const int heights[] = {8, 16, 32, 64};
+    constexpr int NCAND = 12;  // widths x heights
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) {
         if (e0) cudaEventDestroy(e0);
         return b->fail(LBM_ERR_CUDA, "lbm_batch_autotune: events");
     }
     int best_w = b->tile_w, best_h = b->tile_h, rows = 0, rc = LBM_OK;
-    double best = -1.0;
+    double best = -1.0, fine = -1.0;
+    // `n` steps issued by run() and timed: ms per step
+    auto timed = [&](int n, double* ms_per_step, auto run) {
+        cudaError_t e = cudaEventRecord(e0, b->stream);
+        if (e == cudaSuccess) e = run();
+        if (e == cudaSuccess) e = cudaEventRecord(e1, b->stream);
+        if (e == cudaSuccess) e = cudaEventSynchronize(e1);
+        float ms = 0.0f;
+        if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
+        if (e != cudaSuccess) return b->fail(LBM_ERR_CUDA, "lbm_batch_autotune", e);
+        *ms_per_step = ms / n;
+        b->steps += n;
+        for (lbm_handle* h : b->cases) {
+            h->t += n;
+            h->cur = (h->cur + (n & 1)) & 1;
+        }
+        return lbm_batch_sync(b);
+    };
+    // The launches per step first, with one of every candidate's two untimed steps: 2 untimed
+    // and NCAND - 2 timed ones, from a graph as lbm_batch_step has them.
+    std::vector<lbm::BatchTile> tiles;
+    const bool try_fine = !b->limited_waits() && !b->failed && fine_tiling(b, tiles);
+    if (try_fine) {
+        rc = start_per_step(b, tiles);
+        if (rc == LBM_OK) rc = lbm_batch_step(b, 2);
+        if (rc == LBM_OK) {
+            cudaGraphExec_t g = nullptr;
+            cudaError_t e = b->capture_fine(b->steps, NCAND - 2, &g);
+            if (e == cudaSuccess) e = cudaGraphUpload(g, b->stream);
+            rc = e == cudaSuccess ? timed(NCAND - 2, &fine, [&] { return cudaGraphLaunch(g, b->stream); })
+                                  : b->fail(LBM_ERR_CUDA, "lbm_batch_autotune: graph", e);
+            if (g) cudaGraphExecDestroy(g);
+        }
+    }
     for (int w : widths) {
         for (int hgt : heights) {
-            rc = build_tiling(b, w, hgt);
+            if (rc == LBM_OK) rc = build_tiling(b, w, hgt);
             if (rc != LBM_OK) break;
-            rc = lbm_batch_step(b, 2);  // first-touch of the new tables
-            cudaError_t e = rc == LBM_OK ? cudaEventRecord(e0, b->stream) : cudaErrorUnknown;
-            if (e == cudaSuccess) e = b->launch_steps(steps_per_trial);
-            if (e == cudaSuccess) e = cudaEventRecord(e1, b->stream);
-            if (e == cudaSuccess) e = cudaEventSynchronize(e1);
-            float ms = 0.0f;
-            if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
-            if (e != cudaSuccess) { rc = rc != LBM_OK ? rc : b->fail(LBM_ERR_CUDA, "lbm_batch_autotune", e); break; }
-            b->steps += steps_per_trial;
-            for (lbm_handle* h : b->cases) {
-                h->t += steps_per_trial;
-                h->cur = (h->cur + (steps_per_trial & 1)) & 1;
-            }
-            rc = lbm_batch_sync(b);
+            rc = lbm_batch_step(b, try_fine ? 1 : 2);  // first-touch of the new tables
+            double per_step = 0.0;
+            if (rc == LBM_OK) rc = timed(steps_per_trial, &per_step, [&] { return b->launch_steps(steps_per_trial); });
             if (rc != LBM_OK) break;
-            const double per_step = ms / steps_per_trial;
             if (table && rows < table_rows) {
                 table[5 * rows + 0] = w;
                 table[5 * rows + 1] = hgt;
@@ -608,9 +636,28 @@ int lbm_batch_autotune(lbm_batch* b, int32_t steps_per_trial, double* table, int
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (rows_written) *rows_written = rows;
-    if (rc != LBM_OK) return rc;
-    b->want_per_step = false;
-    return build_tiling(b, best_w, best_h);
+    if (rc == LBM_OK) rc = build_tiling(b, best_w, best_h);
+    if (rc != LBM_OK) {
+        b->want_per_step = b->per_step;  // as the failure left it
+        return rc;
+    }
+    b->want_per_step = try_fine && fine <= best;
+    return b->want_per_step ? start_per_step(b, tiles) : LBM_OK;
+}
+
+int lbm_batch_set_per_step(lbm_batch* b, int32_t on) {
+    if (!b) return LBM_ERR_ARG;
+    lbm::detail::DeviceGuard dg(b->device);
+    int rc = LBM_OK;
+    if (on) {
+        std::vector<lbm::BatchTile> tiles;
+        if (!fine_tiling(b, tiles)) return b->fail(LBM_ERR_ARG, "a lattice is too large or too tall for the launches per step");
+        if (!b->per_step && !b->limited_waits()) rc = start_per_step(b, tiles);
+    } else if (b->per_step) {
+        rc = build_tiling(b, b->tile_w, b->tile_h);
+    }
+    if (rc == LBM_OK) b->want_per_step = on != 0;
+    return rc;
 }
 
 int lbm_batch_set_wait_limit(lbm_batch* b, int64_t spin_limit, int32_t hold_tile) {
@@ -620,17 +667,12 @@ int lbm_batch_set_wait_limit(lbm_batch* b, int64_t spin_limit, int32_t hold_tile
     // limited waits are those of the persistent kernel; the defaults give back the launches
     // per step of a batch that had them
     lbm::detail::DeviceGuard dg(b->device);
-    int rc = LBM_OK;
-    if (spin_limit != DEFAULT_SPIN_LIMIT || hold_tile != -1) {
-        if (b->per_step) rc = build_tiling(b, b->tile_w, b->tile_h);
-    } else if (b->want_per_step && !b->per_step) {
-        std::vector<lbm::BatchTile> tiles;
-        if (fine_tiling(b, tiles)) rc = start_per_step(b, tiles);
-    }
-    if (rc != LBM_OK) return rc;
     b->spin_limit = spin_limit;
     b->hold_tile = hold_tile;
     b->drop_graph();
+    if (b->limited_waits()) return b->per_step ? build_tiling(b, b->tile_w, b->tile_h) : LBM_OK;
+    std::vector<lbm::BatchTile> tiles;
+    if (b->want_per_step && !b->per_step && fine_tiling(b, tiles)) return start_per_step(b, tiles);
     return LBM_OK;
 }
 

@@ -103,6 +103,7 @@ def load_library(path: str = LIB_PATH) -> ctypes.CDLL:
         "lbm_batch_set_tiling": (ctypes.c_int, [vp, i32, i32]),
         "lbm_batch_tiling": (ctypes.c_int, [vp] + [ctypes.POINTER(i32)] * 4),
         "lbm_batch_per_step": (ctypes.c_int, [vp]),
+        "lbm_batch_set_per_step": (ctypes.c_int, [vp, i32]),
         "lbm_batch_step": (ctypes.c_int, [vp, i64]),
         "lbm_batch_sync": (ctypes.c_int, [vp]),
         "lbm_batch_autotune": (ctypes.c_int, [vp, i32, ctypes.POINTER(ctypes.c_double), i32,

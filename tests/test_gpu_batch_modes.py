@@ -1,6 +1,7 @@
 """The two ways a batch steps, one launch per step and the persistent kernel: which one
 runs, the way from one to the other, and the same fields as lattices stepped alone."""
 import ctypes
+import json
 
 import pytest
 
@@ -59,4 +60,63 @@ def test_default_waits_leave_the_launches_per_step():
     for s in alone:
         s.step(3 + 4 + 35 + 33 + 6)
     _assert_same(sims, alone, label="modes in turn")
+    b.close()
+
+
+def _us(b, n=96):
+    import torch
+    a, e = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    b.step(n)
+    torch.cuda.synchronize()
+    a.record()
+    b.step(n)
+    e.record()
+    e.synchronize()
+    return a.elapsed_time(e) * 1e3 / n
+
+
+@pytest.mark.parametrize("q", [5, 9])
+def test_a_tuned_batch_is_not_slower_than_it_was(q, tmp_path):
+    # 4 x 64^2: some 3 us a step by launches, some 10 in the best persistent tiling
+    cases = _squares([64] * 4, scalar_q=q)
+    sims, alone = _sims(cases), _sims(cases)
+    b = Batch(sims)
+    before = _us(b)
+    cache = str(tmp_path / "tiles.json")
+    got = b.autotune(steps_per_trial=4, cache=cache)
+    assert got["per_step"] and b.tiling()["per_step"]
+    assert len(got["trials"]) == 12 and all(s.time == 192 + 12 * 6 for s in sims)
+    assert _us(b) < 2 * before
+    for s in alone:
+        s.step(sims[0].time)
+    _assert_same(sims, alone, label="after autotune")
+    # from the cache, on a batch that was moved away, and from a cache without the mode
+    b.set_tiling(32, 4)
+    again = b.autotune(cache=cache)
+    assert again["cached"] and again["per_step"] and b.tiling()["per_step"]
+    known = json.load(open(cache))
+    json.dump({b.signature(): known[b.signature()]}, open(cache, "w"))
+    assert b.autotune(cache=cache)["per_step"]
+    b.set_per_step(False)
+    assert not b.autotune(cache=cache)["per_step"]
+    b.close()
+
+
+def test_a_tuned_batch_with_limited_waits_keeps_the_persistent_kernel():
+    cases = _cases()[:3]
+    sims, alone = _sims(cases), _sims(cases)
+    b = Batch(sims)
+    b.set_wait_limit(1 << 20, -1)
+    got = b.autotune(steps_per_trial=3)
+    assert not got["per_step"] and all(s.time == 60 for s in sims)
+    b.set_per_step(True)  # takes effect with the default waits
+    assert not b.tiling()["per_step"]
+    b.step(3)
+    b.set_wait_limit(1 << 21, -1)
+    assert b.tiling()["per_step"]
+    b.step(3)
+    b.sync()
+    for s in alone:
+        s.step(66)
+    _assert_same(sims, alone, label="limited, then not")
     b.close()
