@@ -120,3 +120,19 @@ def test_a_tuned_batch_with_limited_waits_keeps_the_persistent_kernel():
         s.step(66)
     _assert_same(sims, alone, label="limited, then not")
     b.close()
+
+
+@pytest.mark.parametrize("q", [5, 9])
+def test_ragged_walled_lattices_by_launches(q):
+    cases = [wl.droplet64(nx=nx, ny=ny, R=0.3 * min(nx, ny), scalar_q=q, wall_x=wx, wall_y=wy, rho2=0.5, Fx=1e-6)
+             for nx, ny, wx, wy in ((33, 31, 1, 1), (64, 5, 0, 1), (7, 130, 1, 0), (100, 61, 0, 0), (1, 9, 0, 1), (65, 1, 1, 0))]
+    sims, alone = _sims(cases), _sims(cases)
+    b = Batch(sims)
+    assert b.tiling()["per_step"]
+    b.step(7)
+    b.step(70)  # two graphs of 32 steps from an odd step, six launches
+    b.sync()
+    for s in alone:
+        s.step(77)
+    _assert_same(sims, alone, label="launches per step, D2Q%d" % q)
+    b.close()
