@@ -160,20 +160,25 @@ static int choose_strip_height(const lbm_handle* h) {
 }
 
 // Whether the step runs tiles (tile_kernel, tile64_kernel) instead of strips.  Times
-// are microseconds per step, strips against tiles, on square periodic lattices:
-// (The tiles' launches overlap since: 64^2 takes 2.75 in FP32, 3.4 in bfloat16, 12.7 in
-// FP64; the lines stayed.)
-// * FP64 always: 64^2 82 : 14, 512^2 275 : 165, 1024^2 938 : 622 (D2Q5).  Tiles of 8 x 4
-//   nodes while they leave SMs idle or nearly so (64^2: 13.9 against 15.2 with 16 x 8),
-//   else 16 x 8, whose ring is smaller (128^2: 15.3 against 16.2, 512^2: 165 : 174).
-// * D2Q9 scalars always: the strip kernel spills and holds 34 KB of shared memory per
-//   CTA (FP32 64^2 16.4 : 3.4, 1448^2 191 : 121, 2896^2 704 : 466; bfloat16 64^2 24 : 4.1,
-//   2896^2 563 : 533).
-// * D2Q5 while the strips' serial rows show: FP32 64^2 11.6 : 3.4, 512^2 18.0 : 11.8, 724^2
-//   29.7 : 28.3, then 1024^2 50.7 : 52.3, 2048^2 179 : 194; bfloat16 64^2 20 : 4.0, 512^2
-//   27 : 18, 1024^2 65 : 64, then 1448^2 125 : 126, 2048^2 239 : 246.  Beyond that where
-//   the strips' last 128 columns idle more than the tiles cost (8 %, 16-bit storage 4 %).
-// Tiles address within a row of blocks by 32-bit offsets, and by grid.y.
+// are microseconds per step, strips against tiles with overlapped launches, on square
+// periodic lattices:
+// * FP64 while the offsets below fit: 64^2 81 : 13.2, 512^2 274 : 165, 1024^2 935 : 628
+//   (D2Q5), 512^2 312 : 192 (D2Q9).  Tiles of 8 x 4 nodes while they leave SMs idle or nearly
+//   so (96^2: 13.4 against 14.8 with 16 x 8), else 16 x 8, whose ring is smaller (128^2: 14.8
+//   against 15.3, 512^2: 165 : 174; the two cross near 115^2).
+// * D2Q9 scalars while the offsets fit: the strip kernel spills and holds 34 KB of shared
+//   memory per CTA (FP32 64^2 15.9 : 2.7, 1448^2 191 : 123, 2896^2 705 : 475; bfloat16 64^2
+//   24 : 3.7, 2896^2 558 : 556).
+// * D2Q5 while the strips' serial rows show: FP32 64^2 11.5 : 2.7, 512^2 17.8 : 11.0, 836^2
+//   39.1 : 36.8, and against the tiles 1024^2 50.6 : 51.6, 2048^2 179 : 194; bfloat16 64^2
+//   19.7 : 3.3, 512^2 27 : 17.6, 1225^2 95.6 : 93.7, then 1448^2 124 : 129, 2048^2 237 : 251.  The
+//   lines were taken before the tiles' launches overlapped; in FP32 the two now cross near
+//   950 000 nodes (900^2 43.7 : 42.1, 980^2 49.8 : 48.3), so just above its line the strips cost
+//   3 to 4 %.  Beyond that, tiles where the strips' last 128 columns idle more than the
+//   tiles cost: 8 %, 16-bit storage 4 % (of 1024 rows: FP32 1060 columns, 6 % idle, 57.9 :
+//   54.5; bfloat16 1700, 4 % idle, 104 : 108).
+// Tiles address within a row of blocks by 32-bit offsets, and by grid.y: beyond 2^31 words
+// of populations (FP32 D2Q9 60 M nodes, FP64 D2Q5 77 M) or 262 140 rows everything steps in strips.
 static int choose_tiles(const lbm_handle* h) {
     const lbm_params& p = h->p;
     const long long nx = p.nx, ny = p.ny, nodes = nx * ny;

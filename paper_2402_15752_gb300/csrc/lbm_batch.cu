@@ -2,8 +2,8 @@
 // FP32 lattices, each an lbm_handle of its own, advanced together by the
 // persistent batched kernel (lbm_batch_kernels.cuh) in one cooperative launch
 // per call -- or per 32 steps, replayed from a captured CUDA graph -- with the
-// tile shape chosen by timing candidates (lbm_batch_autotune); or, by default where
-// that is the faster (choose_per_step), by one launch of small tiles per step.
+// tile shape chosen by timing candidates (lbm_batch_autotune); or, where that is the
+// faster (choose_per_step, lbm_batch_autotune), by one launch of small tiles per step.
 #include "lbm.h"
 #include "lbm_handle.h"
 #include "lbm_internal.h"
@@ -423,14 +423,16 @@ int start_per_step(lbm_batch* b, const std::vector<lbm::BatchTile>& tiles) {
     return LBM_OK;
 }
 
-// A batch whose tiling nobody has chosen (set_tiling, autotune) and whose waits nobody has
-// limited steps by one launch per step over tiles of 32 x 4 nodes, unless the persistent
+// A new batch steps by one launch per step over tiles of 32 x 4 nodes, unless the persistent
 // kernel's default 128 x 16 tiles suit it: D2Q5 scalars, at least two tiles per CTA, and
-// lattices that fill the tiles' columns.  Microseconds per step, persistent : per step
-// (D2Q5): 4 lattices of 64^2 32.3 : 2.6, 16 of 96^2 32.7 : 7.3, 64 of 128^2 61.5 : 55.3
-// (fewer tiles than CTAs), 64 of sides 64 .. 512 332 : 307 and 256 of them 1383 : 1313 (a
-// sixth of the columns idle); 64 of 256^2 202 : 208 and 8 of 1024^2 407 : 409 before the
-// steps' launches overlapped.  D2Q9: 64 of 256^2 279 : 254, 8 of 1024^2 567 : 490.
+// lattices that fill the tiles' columns.  Microseconds per step, persistent : per step, with
+// overlapped launches (D2Q5): 4 lattices of 64^2 32.1 : 2.6, 16 of 96^2 32.4 : 7.3, 64 of
+// 128^2 61.0 : 55.3 and 32 of 256^2 124 : 105 (fewer than two tiles per CTA), 64 of uneven
+// sides from 64 to 512 248 : 203 and 256 of them 1049 : 985 (a sixth of the columns idle), 64
+// of 256^2 201 : 206, 8 of 1024^2 405 : 405.  Between two and three tiles per CTA the launches
+// can still be ahead (8 of 640^2 187 : 162; the line is from before they overlapped).
+// D2Q9: 64 of 256^2 278 : 253, 8 of 1024^2 570 : 491.  set_tiling, autotune and set_per_step
+// choose otherwise.
 int choose_per_step(lbm_batch* b) {
     std::vector<lbm::BatchTile> tiles;
     if (!fine_tiling(b, tiles)) return LBM_OK;

@@ -306,13 +306,19 @@ struct Ring {
 // order of a kernel that holds whole units of rows).  So group g of an input row is
 // issued 2 g rows after its first group, when group g - 1 of the next row has been.
 //
-// What bounds it: the 9 MMAs of a row, which one thread issues about every 85 ns (0.75
-// us a row against the 0.55 us of its bytes; a second issuer would have to share the
-// accumulators, whose order of accumulation is kept).  48 -> 48 channels, 16 images of 256 x
-// 256: units of 4 rows loaded with their 2 halo rows as 18 boxes of 4 KB took 54 us
-// (76 at dilation 8, units of 2 rows) and 66 us (77) with the mask epilogue, bound by
-// the TMA's time per box and pixel row; one box of 128-byte pixel slots per row,
-// loaded once: 46 us at every dilation, 52 with the mask epilogue.
+// What bounds it: the MMA warp, a serial chain.  48 -> 48 channels, 16 images of 256 x 256
+// (clock64 in that warp; a CTA lasts 84,000 clocks and takes 54 rows): 14,400 clocks pass
+// before its first MMA (the weights into shared memory, the slots zeroed), then each
+// row takes 1,296: 190 waiting for a free output slot, 190 for an input row (384 and
+// 271 with the mask epilogue) and 917 in the warp's own instructions, about half of them
+// the issue of the nine MMAs, the rest the walk of the three staggered groups and the
+// commits.  The tensor pipe is 42 % active, shared memory (l1tex) 44 % and DRAM 41 % of
+// their peaks, so none of them bounds it.  A second issuer would have to share the
+// accumulators, whose order of accumulation is kept.
+// Units of 4 rows loaded with their 2 halo rows as 18 boxes of 4 KB took 54 us (76 at
+// dilation 8, units of 2 rows) and 66 us (77) with the mask epilogue, bound by the TMA's time
+// per box and pixel row; one box of 128-byte pixel slots per row, loaded once: 46 us at
+// every dilation, 52 with the mask epilogue.
 template <int CI, int CO>
 struct Fw {
     static constexpr int KB = CI / 16;                         // 16-channel groups of the input
