@@ -63,16 +63,18 @@ def test_default_waits_leave_the_launches_per_step():
     b.close()
 
 
-def _us(b, n=96):
+def _us(b, n=32):
+    """us per step, the best of 6 runs of n steps."""
     import torch
-    a, e = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-    b.step(n)
-    torch.cuda.synchronize()
-    a.record()
-    b.step(n)
-    e.record()
-    e.synchronize()
-    return a.elapsed_time(e) * 1e3 / n
+    best = float("inf")
+    for _ in range(6):
+        a, e = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        b.step(n)
+        e.record()
+        e.synchronize()
+        best = min(best, a.elapsed_time(e) * 1e3 / n)
+    return best
 
 
 @pytest.mark.parametrize("q", [5, 9])
